@@ -267,8 +267,8 @@ int32_t stm_energy(stm_ctx *ctx, double *energy);
  * (one class on uniform meshes) time the residual kernels with 64, 128, 256
  * and 512 threads per block, reps times each, on scratch data of the mesh's
  * own layout, and keep the fastest for later applies (before any autotune call
- * a class uses 512 threads where the FP64 passes' shared memory leaves three or
- * fewer blocks per SM, else 256).  Reports per class (up to
+ * a class uses 64 to 512 threads by its work per element, q (p+1)^3, and size).  Reports
+ * per class (up to
  * n_max) the degrees, the chosen block size and its time in ms; *n_out = the
  * number of classes.  Allocates scratch buffers for the duration of the call. */
 int32_t stm_autotune(stm_ctx *ctx, double dt, int32_t reps, int32_t n_max, int32_t *P, int32_t *Q,

@@ -64,6 +64,12 @@ struct Tables {
   T hf[kMaxN];            // dt/2 * sqrt(2a+1)
   T lv[kMaxN];            // sqrt(2a+1)
   T kq[kMaxN];            // -1 / (4 sqrt(2a+1)): folds the flux lift into the curl (k_apply)
+  // unnormalised temporal moments of the two-kernel passes: y_i = ts[i] y'_i with ts[i] = B[i][i]
+  // (i >= 1) or B[0][1], y'_i = u_i + tr[i] u_{i+2} (rows 0 and 1: also + u_1 and u_1 - u_0 in
+  // place of u_i), and lr[j] = sqrt(2j+1) / sqrt(3) of the odd part of a trace
+  T ts[kMaxQ], tr[kMaxQ], lr[kMaxN];
+  // k_apply's line coefficients: the nonzeros of dt D in row order, then -hf[0], -hf[N - 1]
+  T ld[kMaxN * kMaxN / 4 + 2];
 };
 
 template <typename T>
@@ -105,7 +111,8 @@ struct ApplyArgs {
   // local refinement in time (Sec. 2.2): this class's elements split the slab into nk equal
   // sub-intervals (the tables then hold dt / nk); nkl[e] = log2 N_K of every element (null: all 1);
   // tmat: temporal transfer matrices M^{r,o}[a][b] = int_0^1 L_a(s) L_b((o + s) / r) ds for
-  // r = 2, 4, 8 (matrices 0-1, 2-5, 6-13), kMaxQ x kMaxQ each
+  // r = 2, 4, 8 (matrices 0-1, 2-5, 6-13), kMaxQ x kMaxQ each, acting on the unnormalised
+  // moments: entry [a][b] times ts[b] / ts[a], then (matrices 14-27) times ts[a] / (r ts[b])
   int nk = 1;
   const uint8_t* nkl = nullptr;
   const T* tmat = nullptr;
@@ -230,59 +237,101 @@ __host__ __device__ constexpr int residual_max_threads(int P, int Q) {
              : 256;
 }
 
+// Sums and products of the two-kernel passes.  The FP64 pipe of sm_103a issues an FMA with three
+// register operands at 2.0 per clock and SM, but additions, multiplications and FMAs with a
+// constant-bank or immediate operand at 1.68 (measured with register-only chains), and these
+// passes are bound by that pipe.  So in FP64 x + y is fma(x, 1, y), x - y is fma(y, -1, x) and
+// x y is fma(x, y, -0.0), bit for bit the same results, with the constants read from shared memory (where the compiler cannot
+// know them), and every table coefficient comes from shared memory too.
+template <typename T>
+struct PassOps {
+  T one, mone, nzero;
+  __device__ __forceinline__ T add(T x, T y) const { return sizeof(T) == 8 ? fma(x, one, y) : x + y; }
+  // (a negated operand would cost an addition of its own where the negation meets a branch)
+  __device__ __forceinline__ T sub(T x, T y) const { return sizeof(T) == 8 ? fma(y, mone, x) : x - y; }
+  __device__ __forceinline__ T mul(T x, T y) const { return sizeof(T) == 8 ? fma(x, y, nzero) : x * y; }
+};
+
+// Default block of the two-kernel passes, by the element's work per pass: small blocks, so that many
+// elements are in different phases (loads, mass rows, line passes, stores) on an SM, as long as
+// the lines of a pass keep their warps busy.  The lines lie where the autotuner's sweep over
+// p = 1..7, q = 1..4 (FP64, uniform and hp meshes, 64..512 threads) changes its choice; at p = 4,
+// q = 3 (64^3 bricks) 128 threads take 8.55 ms per k_apply against 8.91 ms for 256.  A mesh (or
+// class) of at most two elements per SM (152) waits for one element's own chain of loads, passes
+// and barriers instead: at least 256 threads there (4^3 elements, p = 2, q = 1: 11.6 us per apply
+// against 14.4 us for 64).
+constexpr int residual_default_block(int P, int Q, int64_t n_elem) {
+  const int w = Q * (P + 1) * (P + 1) * (P + 1);
+  const int t = w <= 200 ? 64 : (w <= 380 ? 128 : (w <= 700 ? 256 : 512));
+  const int b = n_elem <= 2 * 152 && t < 256 ? 256 : t;
+  return b < residual_max_threads(P, Q) ? b : residual_max_threads(P, Q);
+}
+
+// Blocks per SM the compiler leaves registers for: 64 registers a thread at the largest block.
+__host__ __device__ constexpr int residual_min_blocks(int P, int Q) { return residual_max_threads(P, Q) == 512 ? 2 : 4; }
+
 // TR: the mesh has elements with N_K > 1 (HP only); false compiles the one-sub-interval code
+//
+// The moments are kept unnormalised, y'_i = y_i / ts[i]: rows 0 and 1 are u_0 + u_1 and u_1 - u_0
+// plus one FMA, row i >= 2 is u_i plus one FMA (2 Q - 2 operations per point at q = 3 instead of
+// the 2 Q + 1 products of B), and k_apply's tables carry ts[i].  A trace takes N operations: the
+// even part, the odd part relative to lv[1], and one FMA per face.  64^3 bricks, p = 4, q = 3,
+// FP64: 6.15 -> 3.6 ms (241 FMA warp instructions per element, the FP64 pipe 0.85 busy).
 template <typename T, int P, int Q, bool HP, bool TR = false>
-__global__ void __launch_bounds__(residual_max_threads(P, Q)) k_prep(ApplyArgs<T> A) {
+__global__ void __launch_bounds__(residual_max_threads(P, Q), residual_min_blocks(P, Q)) k_prep(ApplyArgs<T> A) {
   if (A.skip && *A.skip) return;
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* ys = reinterpret_cast<T*>(smem_raw);  // [2][3][Q][N3]
-  // A P^{-1} v (pinv set, no slab start): the inverse block-diagonal mass scales every unknown
-  // mode of a (field, component) block, so it is folded into that block's B coefficients once
-  // per element (6 (Q+1) Q products) instead of one multiply per coefficient
-  __shared__ T Bsc[6][kMaxQ][kMaxQ + 1];
+  __shared__ T cs[kMaxQ + 2 * kMaxN + 3];  // tr | lv | lr | 1, -1, -0.0
+  T *c_tr = cs, *c_lv = cs + kMaxQ, *c_lr = c_lv + kMaxN;
+  if (threadIdx.x < kMaxQ) c_tr[threadIdx.x] = A.tb.tr[threadIdx.x];
+  if (threadIdx.x < N) {
+    c_lv[threadIdx.x] = A.tb.lv[threadIdx.x];
+    c_lr[threadIdx.x] = A.tb.lr[threadIdx.x];
+  }
+  if (threadIdx.x < 3) c_lr[kMaxN + threadIdx.x] = threadIdx.x == 2 ? -T(0) : (threadIdx.x ? T(-1) : T(1));
+  __syncthreads();
+  const PassOps<T> op{c_lr[kMaxN], c_lr[kMaxN + 1], c_lr[kMaxN + 2]};
   const int nk = TR ? A.nk : 1, QE = TR ? nk * Q : Q;
   for (int64_t blk = blockIdx.x; blk < A.n_elem; blk += gridDim.x) {
     const ElemAddr<T, P, Q, HP, TR> ad(A, blk);
-    if (A.pinv) {
-      for (int it = threadIdx.x; it < 6 * Q * (Q + 1); it += blockDim.x) {
-        const int fc = it / (Q * (Q + 1)), r = it - fc * Q * (Q + 1), i = r / (Q + 1), m = r - i * (Q + 1);
-        Bsc[fc][i][m] = A.tb.B[i][m] * A.pinv[ad.e * 6 + fc];
-      }
-      __syncthreads();
-    }
 #pragma unroll 1
     for (int k = 0; k < nk; ++k) {  // temporal sub-intervals (Sec. 2.2)
-    auto contract = [&](auto prec) {
-      constexpr bool PRE = decltype(prec)::value;
+    // START: the sub-interval has a mode 0 (the slab start, or the end of sub-interval k - 1);
+    // PRE: A P^{-1} v, the inverse block-diagonal mass scales the moments
+    auto contract = [&](auto startc, auto prec) {
+      constexpr bool START = decltype(startc)::value, PRE = decltype(prec)::value;
       for (int it = threadIdx.x; it < 6 * N3; it += blockDim.x) {
         const int fc = it / N3, s = it - fc * N3;
+        const T* um = A.um + ad.um + fc * ad.um_cs + k * Q * N3 + s;
         T u[Q + 1];
-        // mode 0 of sub-interval k: the slab start, else mode 1 (end value) of sub-interval k - 1
-        if (k == 0) u[0] = (!PRE && A.u0) ? A.u0[ad.u0 + fc * ad.u0_cs + s] : T(0);
-        else u[0] = A.um[ad.um + fc * ad.um_cs + (k - 1) * Q * N3 + s];
+        u[0] = T(0);
+        if constexpr (START) u[0] = k == 0 ? A.u0[ad.u0 + fc * ad.u0_cs + s] : um[-N3 * Q];
 #pragma unroll
-        for (int m = 1; m <= Q; ++m) u[m] = A.um[ad.um + fc * ad.um_cs + (k * Q + m - 1) * N3 + s];
+        for (int m = 1; m <= Q; ++m) u[m] = um[(m - 1) * N3];
+        T sc = T(1);
+        if constexpr (PRE) sc = A.pinv[ad.e * 6 + fc];
         T* yg = A.y + ad.R + fc * (int64_t)(QE * N3) + k * Q * N3 + s;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-          T acc = T(0);
-          bool first = true;
-#pragma unroll
-          for (int m = 0; m <= Q; ++m) {
-            if (b_nz(i, m)) {
-              const T bb = PRE ? Bsc[fc][i][m] : A.tb.B[i][m];
-              acc = first ? bb * u[m] : fma(bb, u[m], acc);
-              first = false;
-            }
-          }
+          T acc = i == 0 ? (START ? op.add(u[0], u[1]) : u[1])
+                         : (i == 1 ? (START ? op.sub(u[1], u[0]) : u[1]) : u[i]);
+          if (i + 2 <= Q) acc = fma(c_tr[i], u[i + 2 <= Q ? i + 2 : 0], acc);
+          if constexpr (PRE) acc = op.mul(acc, sc);
           ys[(fc * Q + i) * N3 + s] = acc;
           yg[i * N3] = acc;
         }
       }
     };
-    if (A.pinv) contract(std::true_type{});
-    else contract(std::false_type{});
+    if (A.pinv) {
+      if (k == 0) contract(std::false_type{}, std::true_type{});
+      else contract(std::true_type{}, std::true_type{});
+    } else if (k > 0 || A.u0) {
+      contract(std::true_type{}, std::false_type{});
+    } else {
+      contract(std::false_type{}, std::false_type{});
+    }
     __syncthreads();
     // traces: items (f, a, bi, i, t)
     for (int it = threadIdx.x; it < 12 * Q * N2; it += blockDim.x) {
@@ -296,16 +345,16 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q)) k_prep(ApplyArgs<T
       int base, stride;
       line_geom<N>(a, t, base, stride);
       const T* yl = ys + ((f * 3 + b) * Q + i) * N3 + base;
-      T ev = T(0), od = T(0);
+      T ev = yl[0], od = N > 1 ? yl[stride] : T(0);  // lv[0] = 1; od relative to lv[1]
 #pragma unroll
-      for (int j = 0; j < N; ++j) {
+      for (int j = 2; j < N; ++j) {
         const T v = yl[j * stride];
-        if (j & 1) od = fma(A.tb.lv[j], v, od);
-        else ev = fma(A.tb.lv[j], v, ev);
+        if (j & 1) od = fma(c_lr[j], v, od);
+        else ev = fma(c_lv[j], v, ev);
       }
       const int64_t o = ((((int64_t)f * 3 + a) * 2 + 0) * 2 + bi) * QE + k * Q + i;
-      A.tr[ad.tr + o * N2 + t] = ev - od;                 // face x^_a = 0
-      A.tr[ad.tr + (o + 2 * QE) * N2 + t] = ev + od;      // face x^_a = 1
+      A.tr[ad.tr + o * N2 + t] = N > 1 ? fma(-c_lv[N > 1], od, ev) : ev;            // face x^_a = 0
+      A.tr[ad.tr + (o + 2 * QE) * N2 + t] = N > 1 ? fma(c_lv[N > 1], od, ev) : ev;  // face x^_a = 1
     }
     __syncthreads();
     }
@@ -361,7 +410,7 @@ __device__ __forceinline__ T nbr_trace(const ApplyArgs<T>& A, int64_t en, int ns
   if (nkn == A.nk) return src[(int64_t)(k * qn + i) * nn2];
   if (nkn < A.nk) {
     const int r = A.nk / nkn, kk = k / r, o = k - kk * r;
-    const T* M = A.tmat + tmat_index(r, o) * (kMaxQ * kMaxQ) + i * kMaxQ;
+    const T* M = A.tmat + tmat_index(r, o) * (kMaxQ * kMaxQ) + i * kMaxQ;  // M[i][l] ts[l] / ts[i]
     T acc = T(0);
     for (int l = i; l < qt; ++l) acc = fma(M[l], src[(int64_t)(kk * qn + l) * nn2], acc);
     return acc;
@@ -369,10 +418,10 @@ __device__ __forceinline__ T nbr_trace(const ApplyArgs<T>& A, int64_t en, int ns
   const int r = nkn / A.nk;
   T acc = T(0);
   for (int o = 0; o < r; ++o) {
-    const T* M = A.tmat + tmat_index(r, o) * (kMaxQ * kMaxQ);
+    const T* M = A.tmat + (14 + tmat_index(r, o)) * (kMaxQ * kMaxQ);  // M[j][i] ts[j] / (r ts[i])
     for (int j = 0; j <= i; ++j) acc = fma(M[j * kMaxQ + i], src[(int64_t)((k * r + o) * qn + j) * nn2], acc);
   }
-  return acc / T(r);
+  return acc;
 }
 
 // Offset in the test layout [f][c][QE][N3] of entry w = (c, i, s) of one sub-interval's
@@ -387,27 +436,6 @@ __device__ __forceinline__ int64_t test_ofs(int64_t rk, int f, int w, int QE) {
 // Line passes of k_apply: pass k handles, for output component c, the derivative axis
 // a = (k == 0 ? (c == 0 ? 1 : 0) : (c == 2 ? 1 : 2)).  The line's term carries the sign
 // s_F eps_{cab} (s_E = -1, s_H = +1), negative exactly when (f == 0) == ((c, a) cyclic).
-// curl_combo maps the combination index cb (NF fields x 3 components) to (field slot fl,
-// component c) with the positive lines first, and returns the sign.
-template <int NF>
-__device__ __forceinline__ void curl_combo(int k, int f0, int cb, int& fl, int& c, bool& neg) {
-  if constexpr (NF == 2) {
-    // pass 0: positive (f, c) = (0,1) (1,0) (1,2), negative (0,0) (0,2) (1,1); pass 1: the reverse
-    constexpr int ord[2][6] = {{1, 3, 5, 0, 2, 4}, {0, 2, 4, 1, 3, 5}};
-    const int fc = ord[k][cb];
-    fl = fc / 3;
-    c = fc - 3 * fl;
-    neg = cb >= 3;
-  } else {
-    // one field per pass: (f, pass) = (0,0) and (1,1) have one positive line set, c = 1;
-    // (1,0) and (0,1) have two, c = 0 and 2
-    fl = 0;
-    const bool one = (f0 == k);
-    constexpr int ord1[3] = {1, 0, 2}, ord2[3] = {0, 2, 1};
-    c = one ? ord1[cb] : ord2[cb];
-    neg = one ? cb >= 1 : cb >= 2;
-  }
-}
 
 // Shared memory per k_apply pass: y of the other field and the residual rows;
 // both fields in one pass when that fits in ~110 KB, else one field per pass.
@@ -419,8 +447,34 @@ struct ApplyShape {
   static constexpr size_t smem = sizeof(T) * 2 * NF * 3 * Q * N3;
 };
 
+// Position of the nonzero D[a][b] (d_nz) of an N x N table in row order; d_count<N>(N, 0) of them.
+template <int N>
+__host__ __device__ constexpr int d_count(int a, int b) {
+  int k = 0;
+  for (int x = 0; x < N; ++x)
+    for (int y = 0; y < N; ++y) {
+      if (x == a && y == b) return k;
+      k += d_nz(x, y) ? 1 : 0;
+    }
+  return k;
+}
+
+// k_apply's coefficients in shared memory, per sign of the line's curl term and temporal mode i
+// (they carry ts[i], the moments being unnormalised): the ND nonzeros of dt D, then the flux-lift
+// factors -dt/2 lv of rows 0 and N - 1.
+template <typename T, int P, int Q>
+struct LineTab {
+  static constexpr int N = P + 1, ND = d_count<N>(N, 0), W = ND + 2;
+  T c[2][Q][W];
+  T kq[N], one, mone, nzero, ts[Q];
+};
+
+// FP64 pipe bound like k_prep (486 FMA warp instructions per element at p = 4, q = 3).  The line's
+// sign is in its coefficients, so a warp never runs both signs, and the mass rows load all their
+// modes before the first product.  64^3 bricks, p = 4, q = 3, FP64: 10.27 -> 8.55 ms; without the
+// trace loads of the line passes it takes 7.5 ms, with all memory traffic hitting L2 8.4 ms.
 template <typename T, int P, int Q, bool HP, bool TR = false>
-__global__ void __launch_bounds__(residual_max_threads(P, Q)) k_apply(ApplyArgs<T> A) {
+__global__ void __launch_bounds__(residual_max_threads(P, Q), residual_min_blocks(P, Q)) k_apply(ApplyArgs<T> A) {
   if (A.skip && *A.skip) return;
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   constexpr int NF = ApplyShape<T, P, Q>::NF;
@@ -429,13 +483,30 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q)) k_apply(ApplyArgs<
   T* ys = reinterpret_cast<T*>(smem_raw);  // [NF][3][Q][N3]: y of the other field
   T* Rs = ys + NF * FB;                     // [NF][3][Q][N3]: residual rows
   __shared__ FaceCache fcs;                 // uneven degrees only
+  __shared__ int nb[6];                     // the element's neighbours
+  using LT = LineTab<T, P, Q>;
+  __shared__ LT lt;
+  for (int it = threadIdx.x; it < 2 * Q * LT::W; it += blockDim.x) {
+    const int w = it % LT::W, i = (it / LT::W) % Q;
+    const T v = A.tb.ts[i] * A.tb.ld[w];
+    (&lt.c[0][0][0])[it] = it < Q * LT::W ? v : -v;
+  }
+  if (threadIdx.x < Q) lt.ts[threadIdx.x] = A.tb.ts[threadIdx.x];
+  if (threadIdx.x < N) lt.kq[threadIdx.x] = A.tb.kq[threadIdx.x];
+  if (threadIdx.x == 0) {
+    lt.one = T(1);
+    lt.mone = T(-1);
+    lt.nzero = -T(0);
+  }
+  __syncthreads();
+  const PassOps<T> op_{lt.one, lt.mone, lt.nzero};
   const int nk = TR ? A.nk : 1, QE = TR ? nk * Q : Q;
   for (int64_t blk = blockIdx.x; blk < A.n_elem; blk += gridDim.x) {
     const ElemAddr<T, P, Q, HP, TR> ad(A, blk);
     const int64_t e = ad.e;
-    const int32_t* nb = A.nbr + e * 6;
+    if (threadIdx.x < 6) nb[threadIdx.x] = A.nbr[e * 6 + threadIdx.x];
     if (HP && threadIdx.x < 6) {  // read after the first barrier below
-      const int f = threadIdx.x, en = nb[f];
+      const int f = threadIdx.x, en = A.nbr[e * 6 + f];
       fcs.off[f] = en >= 0 ? A.off_tr[en] : (en == -2 ? A.hoff[A.hslot[e * 6 + f]] : 0);
       fcs.pq[f] = en >= 0 ? A.pq[en] : 0;
       fcs.nk[f] = (en >= 0 && A.nkl) ? 1 << A.nkl[en] : 1;
@@ -449,6 +520,29 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q)) k_apply(ApplyArgs<
         const int fl = NF == 1 ? 0 : it / FB;
         ys[it] = A.y[test_ofs<Q, N3, TR>(rk, 1 - (f0 + fl), it - fl * FB, QE)];
       }
+      // the traces of line `it` of pass k: own (xm, xp) and the other side's (om, op) of the
+      // tangential component b of the other field on the two faces normal to a
+      auto line_traces = [&](int k, int it, T& xm, T& xp, T& om, T& op) {
+        const int cb = it / (Q * N2), r = it - cb * (Q * N2);
+        const int i = r / N2, t = r - i * N2;
+        const int fl = NF == 1 ? 0 : cb / 3, c = cb - 3 * fl, fp = 1 - (f0 + fl);
+        const int a = (k == 0) ? (c == 0 ? 1 : 0) : (c == 2 ? 1 : 2);
+        const int b = 3 - c - a;
+        const int bi = (a == 0) ? b - 1 : (a == 1 ? b / 2 : b);
+        const int64_t so = ((((int64_t)fp * 3 + a) * 2) * 2 + bi) * QE + sk * Q + i;  // side-0 slot
+        const T* tre = A.tr + ad.tr;
+        xm = tre[so * N2 + t];
+        xp = tre[(so + 2 * QE) * N2 + t];
+        const int ep = nb[2 * a + 1], em = nb[2 * a];
+        // the neighbour's trace, or on a PEC face the mirror value (E: -own, so the jump is
+        // 2 own; H: +own, jump 0) chosen by integer ops
+        if (ep >= 0) op = nbr_trace<T, N, Q, HP, TR>(A, ep, 0, fp, a, bi, i, t, sk, fcs, 2 * a + 1);
+        else if (HP && ep == -2) op = A.hbuf[fcs.off[2 * a + 1] + ((fp * 2 + bi) * Q + i) * N2 + t];
+        else op = (fp == 0) ? neg_bits(xp) : xp;
+        if (em >= 0) om = nbr_trace<T, N, Q, HP, TR>(A, em, 1, fp, a, bi, i, t, sk, fcs, 2 * a);
+        else if (HP && em == -2) om = A.hbuf[fcs.off[2 * a] + ((fp * 2 + bi) * Q + i) * N2 + t];
+        else om = (fp == 0) ? neg_bits(xm) : xm;
+      };
       // mass rows: items (field, component, s), the temporal modes unrolled; the variant
       // (mode 0 of the sub-interval, preconditioned input, load) is chosen once per pass so
       // no FP64 instruction is predicated
@@ -463,18 +557,22 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q)) k_apply(ApplyArgs<
           const T* uc = A.um + ad.um + fc * ad.um_cs + (int64_t)sk * Q * N3 + s;
           T* Rr = Rs + fl * FB + cc * Q * N3 + s;
           // with PRE (A P^{-1} v) the mass block times P^{-1} is the identity: the term is v
-          {  // mode 0: minus mode 0 of the sub-interval (previous sub-interval's end or slab start)
-            T v = PRE ? uc[0] : mc * uc[0];
-            if constexpr (PREV == 1) v = PRE ? v - uc[-Q * N3] : fma(-mc, uc[-Q * N3], v);
-            if constexpr (PREV == 2) v = fma(-mc, A.u0[ad.u0 + fc * ad.u0_cs + s], v);
-            if constexpr (LOAD) v -= A.b[test_ofs<Q, N3, TR>(rk, f0 + fl, cc * Q * N3 + s, QE)];
-            Rr[0] = v;
+          T v[Q], prevv = T(0);
+#pragma unroll
+          for (int i = 0; i < Q; ++i) v[i] = uc[i * N3];
+          if constexpr (PREV == 1) prevv = uc[-Q * N3];
+          if constexpr (PREV == 2) prevv = A.u0[ad.u0 + fc * ad.u0_cs + s];
+          T bv[Q];
+          if constexpr (LOAD) {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) bv[i] = A.b[test_ofs<Q, N3, TR>(rk, f0 + fl, (cc * Q + i) * N3 + s, QE)];
           }
-#pragma unroll 1
-          for (int i = 1; i < Q; ++i) {
-            T v = PRE ? uc[i * N3] : mc * uc[i * N3];
-            if constexpr (LOAD) v -= A.b[test_ofs<Q, N3, TR>(rk, f0 + fl, (cc * Q + i) * N3 + s, QE)];
-            Rr[i * N3] = v;
+#pragma unroll
+          for (int i = 0; i < Q; ++i) {
+            T w = PRE ? v[i] : op_.mul(mc, v[i]);
+            if (i == 0 && PREV != 0) w = PRE ? op_.sub(w, prevv) : fma(-mc, prevv, w);
+            if constexpr (LOAD) w = op_.sub(w, bv[i]);
+            Rr[i * N3] = w;
           }
         }
       };
@@ -532,93 +630,73 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q)) k_apply(ApplyArgs<
 #pragma unroll 1
       for (int k = 0; k < 2; ++k) {
         for (int it = threadIdx.x; it < NF * 3 * Q * N2; it += blockDim.x) {
-          // lines ordered by the sign of their curl term, so that a warp rarely holds both
           const int cb = it / (Q * N2), r = it - cb * (Q * N2);
           const int i = r / N2, t = r - i * N2;
-          int fl, c;
-          bool neg;
-          curl_combo<NF>(k, f0, cb, fl, c, neg);
-          const int f = f0 + fl, fp = 1 - f;
+          const int fl = NF == 1 ? 0 : cb / 3, c = cb - 3 * fl;
+          const int f = f0 + fl;
           const int a = (k == 0) ? (c == 0 ? 1 : 0) : (c == 2 ? 1 : 2);
+          const bool neg = (f == 0) == ((a == 0 && c == 2) || a == c + 1);
           const int b = 3 - c - a;
-          const int bi = (a == 0) ? b - 1 : (a == 1 ? b / 2 : b);
           int base, stride;
           line_geom<N>(a, t, base, stride);
           const T* yl = ys + fl * FB + (b * Q + i) * N3 + base;
-          // jumps of the tangential component b of field fp on the faces normal to a
-          const int64_t so = ((((int64_t)fp * 3 + a) * 2) * 2 + bi) * QE + sk * Q + i;  // side-0 slot
-          const T* tre = A.tr + ad.tr;
-          const T xm = tre[so * N2 + t];
-          const T xp = tre[(so + 2 * QE) * N2 + t];
-          const int ep = nb[2 * a + 1], em = nb[2 * a];
-          // the other side's trace: the neighbour's, or on a PEC face the mirror value (E: -own,
-          // so the jump is 2 own; H: +own, jump 0) chosen by integer ops; one subtraction each
-          T op, om;
-          if (ep >= 0) op = nbr_trace<T, N, Q, HP, TR>(A, ep, 0, fp, a, bi, i, t, sk, fcs, 2 * a + 1);
-          else if (HP && ep == -2) op = A.hbuf[fcs.off[2 * a + 1] + ((fp * 2 + bi) * Q + i) * N2 + t];
-          else op = (fp == 0) ? neg_bits(xp) : xp;
-          if (em >= 0) om = nbr_trace<T, N, Q, HP, TR>(A, em, 1, fp, a, bi, i, t, sk, fcs, 2 * a);
-          else if (HP && em == -2) om = A.hbuf[fcs.off[2 * a] + ((fp * 2 + bi) * Q + i) * N2 + t];
-          else om = (fp == 0) ? neg_bits(xm) : xm;
-          const T jp = xp - op, jm = xm - om;
-          const T sp = jp + jm, dm = jp - jm;
+          T xm, xp, om, op;
+          line_traces(k, it, xm, xp, om, op);
+          const T jp = op_.sub(xp, op), jm = op_.sub(xm, om);
+          const T sp = op_.add(jp, jm), dm = op_.sub(jp, jm);
           T yv[N];
 #pragma unroll
           for (int j = 0; j < N; ++j) yv[j] = yl[j * stride];
           T* Rl = Rs + fl * FB + (c * Q + i) * N3 + base;
-          // the sign s_F eps_{cab} of the line's curl and flux terms is a compile-time constant
-          // of each branch, carried by the table operands of the FMAs (no extra instruction);
-          // lines are ordered by sign, so only the warp at the boundary runs both branches
-          auto body = [&](auto negc) {
-            constexpr T sg = decltype(negc)::value ? T(-1) : T(1);
-            if (A.kap) {
-              // D_h: alpha-weighted jumps of component c of the same field f on the two
-              // faces normal to a, lifted with L_al(1) and L_al(0) = (-1)^al L_al(1);
-              // on a PEC face the E jump is the own trace (E - g, g in the load)
-              const int bc = (a == 0) ? c - 1 : (a == 1 ? c / 2 : c);
-              const int64_t sc = ((((int64_t)f * 3 + a) * 2) * 2 + bc) * QE + sk * Q + i;
-              const T zm = tre[sc * N2 + t], zp = tre[(sc + 2 * QE) * N2 + t];
-              // other side: the neighbour's trace; on a PEC face 0 for E (jump = own) and own for H
-              const T gop = (ep >= 0) ? nbr_trace<T, N, Q, HP, TR>(A, ep, 0, f, a, bc, i, t, sk, fcs, 2 * a + 1)
-                                      : (f == 0 ? T(0) : zp);
-              const T gom = (em >= 0) ? nbr_trace<T, N, Q, HP, TR>(A, em, 1, f, a, bc, i, t, sk, fcs, 2 * a)
-                                      : (f == 0 ? T(0) : zm);
-              const T gp = zp - gop, gm = zm - gom;
-              const T* kp = A.kap + e * 24 + f * 12 + 4 * a + bc;
-              const T dp = A.dt_k * kp[2] * gp, dn = A.dt_k * kp[0] * gm;
-              // the central-flux lift hf[al] = (dt/2) lv[al] shares the factor lv[al]
-              const T zev = fma(-sg * A.tb.hf[0], dm, dp + dn), zod = fma(-sg * A.tb.hf[0], sp, dp - dn);
+          const T* lc = lt.c[neg ? 1 : 0][i];  // the sign s_F eps_{cab} is in the coefficients
+          if (A.kap) {
+            // D_h: alpha-weighted jumps of component c of the same field f on the two
+            // faces normal to a, lifted with L_al(1) and L_al(0) = (-1)^al L_al(1);
+            // on a PEC face the E jump is the own trace (E - g, g in the load)
+            const int bc = (a == 0) ? c - 1 : (a == 1 ? c / 2 : c);
+            const int64_t sc = ((((int64_t)f * 3 + a) * 2) * 2 + bc) * QE + sk * Q + i;
+            const T* tre = A.tr + ad.tr;
+            const int ep = nb[2 * a + 1], em = nb[2 * a];
+            const T zm = tre[sc * N2 + t], zp = tre[(sc + 2 * QE) * N2 + t];
+            // other side: the neighbour's trace; on a PEC face 0 for E (jump = own) and own for H
+            const T gop = (ep >= 0) ? nbr_trace<T, N, Q, HP, TR>(A, ep, 0, f, a, bc, i, t, sk, fcs, 2 * a + 1)
+                                    : (f == 0 ? T(0) : zp);
+            const T gom = (em >= 0) ? nbr_trace<T, N, Q, HP, TR>(A, em, 1, f, a, bc, i, t, sk, fcs, 2 * a)
+                                    : (f == 0 ? T(0) : zm);
+            const T gp = op_.sub(zp, gop), gm = op_.sub(zm, gom);
+            const T* kp = A.kap + e * 24 + f * 12 + 4 * a + bc;
+            const T dts = A.dt_k * lt.ts[i];
+            const T dp = dts * kp[2] * gp, dn = dts * kp[0] * gm;
+            // the central-flux lift hf[al] = (dt/2) lv[al] shares the factor lv[al]
+            const T zev = fma(lc[LT::ND], dm, op_.add(dp, dn)), zod = fma(lc[LT::ND], sp, op_.sub(dp, dn));
 #pragma unroll
-              for (int al = 0; al < N; ++al) {
-                T r2 = Rl[al * stride];
-                r2 = fma(A.tb.lv[al], (al & 1) ? zod : zev, r2);
+            for (int al = 0; al < N; ++al) {
+              T r2 = Rl[al * stride];
+              r2 = fma(A.tb.lv[al], (al & 1) ? zod : zev, r2);
 #pragma unroll
-                for (int be = 0; be < N; ++be)
-                  if (d_nz(al, be)) r2 = fma(sg * A.tb.Dt[al][be], yv[be], r2);
-                Rl[al * stride] = r2;
-              }
-            } else {
-              // Dt[a][b] = 2 dt L_a(1) L_b(1) and hf[a] = dt/2 L_a(1) share the factor L_a(1), so
-              // the lift -hf[a] X of every row a but the last equals Dt[a][B] X kq[B] with B the
-              // largest index of the other parity (which every such row's curl sum reaches):
-              // folded into y[B] once per line instead of one FMA per row
-              constexpr int B0 = ((N - 1) & 1) ? N - 1 : N - 2;  // largest odd index: even rows, X = dm
-              constexpr int B1 = ((N - 1) & 1) ? N - 2 : N - 1;  // largest even index: odd rows, X = sp
-              if constexpr (B0 >= 1) yv[B0] = fma(A.tb.kq[B0], dm, yv[B0]);
-              if constexpr (B1 >= 2) yv[B1] = fma(A.tb.kq[B1], sp, yv[B1]);
-#pragma unroll
-              for (int al = 0; al < N; ++al) {
-                T r2 = Rl[al * stride];
-                if (al == N - 1) r2 = fma(-sg * A.tb.hf[al], (al & 1) ? sp : dm, r2);
-#pragma unroll
-                for (int be = 0; be < N; ++be)
-                  if (d_nz(al, be)) r2 = fma(sg * A.tb.Dt[al][be], yv[be], r2);
-                Rl[al * stride] = r2;
-              }
+              for (int be = 0; be < N; ++be)
+                if (d_nz(al, be)) r2 = fma(lc[d_count<N>(al, be)], yv[be], r2);
+              Rl[al * stride] = r2;
             }
-          };
-          if (neg) body(std::true_type{});
-          else body(std::false_type{});
+          } else {
+            // Dt[a][b] = 2 dt L_a(1) L_b(1) and hf[a] = dt/2 L_a(1) share the factor L_a(1), so
+            // the lift -hf[a] X of every row a but the last equals Dt[a][B] X kq[B] with B the
+            // largest index of the other parity (which every such row's curl sum reaches):
+            // folded into y[B] once per line instead of one FMA per row
+            constexpr int B0 = ((N - 1) & 1) ? N - 1 : N - 2;  // largest odd index: even rows, X = dm
+            constexpr int B1 = ((N - 1) & 1) ? N - 2 : N - 1;  // largest even index: odd rows, X = sp
+            if constexpr (B0 >= 1) yv[B0] = fma(lt.kq[B0], dm, yv[B0]);
+            if constexpr (B1 >= 2) yv[B1] = fma(lt.kq[B1], sp, yv[B1]);
+#pragma unroll
+            for (int al = 0; al < N; ++al) {
+              T r2 = Rl[al * stride];
+              if (al == N - 1) r2 = fma(lc[LT::ND + 1], (al & 1) ? sp : dm, r2);
+#pragma unroll
+              for (int be = 0; be < N; ++be)
+                if (d_nz(al, be)) r2 = fma(lc[d_count<N>(al, be)], yv[be], r2);
+              Rl[al * stride] = r2;
+            }
+          }
         }
         __syncthreads();
       }

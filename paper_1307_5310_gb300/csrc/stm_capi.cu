@@ -57,7 +57,7 @@ int launch_residual_ph(int P, int Q, const ApplyArgs<T>& a, cudaStream_t s, int 
 
 template <typename T>
 int launch_residual(int P, int Q, const ApplyArgs<T>& a, cudaStream_t s, int grid, const LaunchEvents& ev) {
-  return launch_residual_ph<T>(P, Q, a, s, grid, ev, 0, 256);
+  return launch_residual_ph<T>(P, Q, a, s, grid, ev, 0, residual_default_block(P, Q, a.n_elem));
 }
 
 // 1-D tables from their closed forms (Sec. 5.1-5.2): B_im = int L_i l_m with
@@ -82,13 +82,25 @@ Tables<T> make_tables(int P, int Q, double dt) {
   }
   for (int i = 0; i < kMaxQ; ++i)
     for (int m = 0; m <= kMaxQ; ++m) t.B[i][m] = (T)B[i][m];
+  for (int i = 0; i < kMaxQ; ++i) {
+    const double si = i == 0 ? 0.5 : 0.5 / (std::sqrt(2.0 * i - 1) * std::sqrt(2.0 * i + 1));  // B[0][1], B[i][i]
+    t.ts[i] = (T)si;
+    t.tr[i] = (i + 2 <= Q && i + 2 <= kMaxQ) ? (T)(B[i][i + 2] / si) : T(0);
+  }
   for (int a = 0; a < N; ++a) {
+    t.lr[a] = (T)(std::sqrt(2.0 * a + 1) / std::sqrt(3.0));
     t.lv[a] = (T)std::sqrt(2.0 * a + 1);
     t.kq[a] = (T)(-0.25 / std::sqrt(2.0 * a + 1));
     t.hf[a] = (T)(0.5 * dt * std::sqrt(2.0 * a + 1));
     for (int b = 0; b < N; ++b)
       if (d_nz(a, b)) t.Dt[a][b] = (T)(dt * 2.0 * std::sqrt(2.0 * a + 1) * std::sqrt(2.0 * b + 1));
   }
+  int w = 0;
+  for (int a = 0; a < N; ++a)
+    for (int b = 0; b < N; ++b)
+      if (d_nz(a, b)) t.ld[w++] = t.Dt[a][b];
+  t.ld[w++] = -t.hf[0];
+  t.ld[w++] = -t.hf[N - 1];
   return t;
 }
 
@@ -477,11 +489,6 @@ int check_wait_err(stm_ctx* c) {
   }
   return h ? fail(c, STM_ETIMEOUT, "FP32 Krylov kernel: a bounded wait on its copies ran out") : STM_OK;
 }
-
-// Default threads per block of the two-kernel residual passes of degree (P, Q): the kernels'
-// largest block (residual_max_threads: 512 where shared memory limits the blocks per SM, else
-// 256).  The autotuner may replace it.
-int default_block(int P, int Q) { return residual_max_threads(P, Q); }
 
 template <typename T>
 int apply(stm_ctx* c, double dt, const T* um, int um_layout, const T* u0, int u0_layout, const T* b, T* R,
@@ -1461,7 +1468,7 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
   c->ne = m->n_elem;
   c->P = m->p[0];
   c->Q = m->q[0];
-  c->block = default_block(c->P, c->Q);
+  c->block = residual_default_block(c->P, c->Q, m->n_elem);
   c->h_p.resize(c->ne);
   c->h_q.resize(c->ne);
   for (int64_t e = 0; e < c->ne; ++e) {
@@ -1841,7 +1848,7 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
         for (int lk = 0; lk < 4 && okh; ++lk) {
           const auto& L = lists[(pp * (kMaxQ + 1) + qq) * 4 + lk];
           if (L.empty()) continue;
-          stm_ctx::Class cl{pp, qq, (int64_t)L.size(), nullptr, default_block(pp, qq)};
+          stm_ctx::Class cl{pp, qq, (int64_t)L.size(), nullptr, residual_default_block(pp, qq, (int64_t)L.size())};
           cl.NK = 1 << lk;
           okh = cudaMalloc(&cl.elist, L.size() * sizeof(int32_t)) == cudaSuccess;
           if (okh) cudaMemcpy(cl.elist, L.data(), L.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
@@ -1852,7 +1859,7 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
       // int_0^1 L_a(s) L_b((o + s) / r) ds by Gauss quadrature (exact: degree <= 2 kMaxQ)
       std::vector<uint8_t> nkl(c->ne);
       for (int64_t e = 0; e < c->ne; ++e) nkl[e] = (uint8_t)lg2(c->h_nk[e]);
-      std::vector<double> tm(14 * kMaxQ * kMaxQ, 0.0), xg, wg;
+      std::vector<double> tm(28 * kMaxQ * kMaxQ, 0.0), xg, wg;
       gauss01(kMaxQ + 1, xg, wg);
       for (int r = 2; r <= 8; r *= 2)
         for (int oo = 0; oo < r; ++oo)
@@ -1863,6 +1870,16 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
             for (int aa = 0; aa < kMaxQ; ++aa)
               for (int bb = 0; bb < kMaxQ; ++bb) tm[(tmat_index(r, oo) * kMaxQ + aa) * kMaxQ + bb] += wg[g] * La[aa] * Lb[bb];
           }
+      // scaled to the unnormalised moments of the kernels: own finer (0-13), own coarser (14-27)
+      const Tables<double> tb = make_tables<double>(0, kMaxQ, 1.0);
+      for (int r = 2; r <= 8; r *= 2)
+        for (int oo = 0; oo < r; ++oo)
+          for (int aa = 0; aa < kMaxQ; ++aa)
+            for (int bb = 0; bb < kMaxQ; ++bb) {
+              double* M = &tm[(tmat_index(r, oo) * kMaxQ + aa) * kMaxQ + bb];
+              M[14 * kMaxQ * kMaxQ] = *M * tb.ts[aa] / (r * tb.ts[bb]);
+              *M *= tb.ts[bb] / tb.ts[aa];
+            }
       std::vector<float> tm32(tm.begin(), tm.end());
       okh = cudaMalloc(&c->nkl, c->ne) == cudaSuccess &&
             cudaMalloc(&c->tmat64, tm.size() * sizeof(double)) == cudaSuccess &&
