@@ -609,7 +609,7 @@ def leg_curved_slabs(slabs=50, ps=(3, 5, 7)):
     """The curved configuration as stated: 32^3 trilinear hexes (vertices moved by 0.1 h sin sin
     sin), p in {3, 5, 7}, q = p - 1, eps = mu = 1, a Gaussian current pulse (width 0.05, centre of
     the domain, Gaussian in time), dt = h/(2p+1), `slabs` mixed-precision slab solves (FP32
-    inner GMRES with the mass term on the tensor cores, FP64 outer refinement) to 1e-9."""
+    inner GMRES, FP64 outer refinement) to 1e-9."""
     from paper_1307_5310_gb300 import meshgen, stm
 
     out = {"workload": f"32^3 trilinear hexes (0.1 h sin sin sin), q = p - 1, Gaussian J (sigma_x = 0.05 at the "

@@ -34,9 +34,10 @@ def _units():
     units = []
     for p in range(8):
         units.append(("residual_inst.cu", f"residual_p{p}.o", [f"-DSTM_P={p}"]))
-    for src in ("krylov.cu", "stm_capi.cu", "stm_noalloc.cu", "load.cu", "curved.cu", "curved_tc.cu", "hp.cu",
-                "server.cu"):
+    for src in ("krylov.cu", "stm_capi.cu", "stm_noalloc.cu", "load.cu", "curved.cu", "hp.cu", "server.cu"):
         units.append((src, src.replace(".cu", ".o"), []))
+    for t in ("float", "double"):
+        units.append(("curved_mass.cu", f"curved_mass_{t}.o", [f"-DSTM_MASS_T={t}"]))
     return units
 
 

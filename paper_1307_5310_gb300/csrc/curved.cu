@@ -95,100 +95,6 @@ __global__ void __launch_bounds__(256) k_metric(const double* __restrict__ X8g, 
   }
 }
 
-template <typename T, int P, int Q>
-__global__ void __launch_bounds__(256) k_mass_curved(const T* __restrict__ um, int64_t um_es, int64_t um_cs,
-                                                     const T* __restrict__ u0, int64_t u0_es, int64_t u0_cs,
-                                                     const T* __restrict__ Gw, const T* __restrict__ eps,
-                                                     const T* __restrict__ mu, CTab<T> L, int64_t ne,
-                                                     T* __restrict__ R, const int32_t* skip) {
-  if (skip && *skip) return;
-  constexpr int N = P + 1, NQ = P + 2, N2 = N * N, N3 = N2 * N, NQ2 = NQ * NQ, NQ3 = NQ2 * NQ;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* g6 = reinterpret_cast<T*>(smem_raw);  // [6][NQ3]
-  T* b0 = g6 + 6 * NQ3;                     // [3][NQ3]
-  T* b1 = b0 + 3 * NQ3;                     // [3][NQ3]
-  for (int64_t e = blockIdx.x; e < ne; e += gridDim.x) {
-    for (int it = threadIdx.x; it < 6 * NQ3; it += blockDim.x) g6[it] = Gw[e * 6 * NQ3 + it];
-#pragma unroll 1
-    for (int f = 0; f < 2; ++f) {
-      const T mat = f == 0 ? eps[e] : mu[e];
-#pragma unroll 1
-      for (int i = 0; i < Q; ++i) {
-        for (int it = threadIdx.x; it < 3 * N3; it += blockDim.x) {
-          const int c = it / N3, s = it - c * N3, fc = f * 3 + c;
-          T v = um[e * um_es + fc * um_cs + i * N3 + s];
-          if (i == 0 && u0) v -= u0[e * u0_es + fc * u0_cs + s];
-          b0[c * NQ3 + s] = v;
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * N2 * NQ; it += blockDim.x) {  // x: j -> gx
-          const int gx = it % NQ, lk = (it / NQ) % N2, c = it / (NQ * N2);
-          const T* in = b0 + c * NQ3 + lk * N;
-          T acc = T(0);
-#pragma unroll
-          for (int j = 0; j < N; ++j) acc = fma(in[j], L.Lq[j][gx], acc);
-          b1[c * NQ3 + lk * NQ + gx] = acc;
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * N * NQ2; it += blockDim.x) {  // y: k -> gy
-          const int gx = it % NQ, gy = (it / NQ) % NQ, l = (it / NQ2) % N, c = it / (NQ2 * N);
-          const T* in = b1 + c * NQ3 + l * N * NQ + gx;
-          T acc = T(0);
-#pragma unroll
-          for (int k = 0; k < N; ++k) acc = fma(in[k * NQ], L.Lq[k][gy], acc);
-          b0[c * NQ3 + (l * NQ + gy) * NQ + gx] = acc;
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * NQ3; it += blockDim.x) {  // z: l -> gz
-          const int g2 = it % NQ2, gz = (it / NQ2) % NQ, c = it / NQ3;
-          const T* in = b0 + c * NQ3 + g2;
-          T acc = T(0);
-#pragma unroll
-          for (int l = 0; l < N; ++l) acc = fma(in[l * NQ2], L.Lq[l][gz], acc);
-          b1[c * NQ3 + gz * NQ2 + g2] = acc;
-        }
-        __syncthreads();
-        for (int g = threadIdx.x; g < NQ3; g += blockDim.x) {  // pointwise w_g G(x_g)
-          const T vx = b1[g], vy = b1[NQ3 + g], vz = b1[2 * NQ3 + g];
-          const T gxx = g6[g], gyy = g6[NQ3 + g], gzz = g6[2 * NQ3 + g];
-          const T gxy = g6[3 * NQ3 + g], gxz = g6[4 * NQ3 + g], gyz = g6[5 * NQ3 + g];
-          b0[g] = mat * fma(gxx, vx, fma(gxy, vy, gxz * vz));
-          b0[NQ3 + g] = mat * fma(gxy, vx, fma(gyy, vy, gyz * vz));
-          b0[2 * NQ3 + g] = mat * fma(gxz, vx, fma(gyz, vy, gzz * vz));
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * N * NQ2; it += blockDim.x) {  // z: gz -> l
-          const int g2 = it % NQ2, l = (it / NQ2) % N, c = it / (NQ2 * N);
-          const T* in = b0 + c * NQ3 + g2;
-          T acc = T(0);
-#pragma unroll
-          for (int gz = 0; gz < NQ; ++gz) acc = fma(in[gz * NQ2], L.Lq[l][gz], acc);
-          b1[c * NQ3 + l * NQ2 + g2] = acc;
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * N2 * NQ; it += blockDim.x) {  // y: gy -> k
-          const int gx = it % NQ, k = (it / NQ) % N, l = (it / (NQ * N)) % N, c = it / (NQ * N2);
-          const T* in = b1 + c * NQ3 + l * NQ2 + gx;
-          T acc = T(0);
-#pragma unroll
-          for (int gy = 0; gy < NQ; ++gy) acc = fma(in[gy * NQ], L.Lq[k][gy], acc);
-          b0[c * NQ3 + (l * N + k) * NQ + gx] = acc;
-        }
-        __syncthreads();
-        for (int it = threadIdx.x; it < 3 * N3; it += blockDim.x) {  // x: gx -> j, write
-          const int j = it % N, lk = (it / N) % N2, c = it / N3;
-          const T* in = b0 + c * NQ3 + lk * NQ;
-          T acc = T(0);
-#pragma unroll
-          for (int gx = 0; gx < NQ; ++gx) acc = fma(in[gx], L.Lq[j][gx], acc);
-          R[(e * 6 + f * 3 + c) * (int64_t)(Q * N3) + i * N3 + lk * N + j] = acc;
-        }
-        __syncthreads();
-      }
-    }
-  }
-}
-
 template <typename S, typename X, bool Add>
 __global__ void k_precond_curved(X* __restrict__ out, const S* __restrict__ V, int64_t ldv, int k, Coef16 y,
                                  const S* __restrict__ Pinv, int64_t qn3, int64_t ne, const int32_t* skip,
@@ -298,37 +204,6 @@ int launch_metric(int P, const double* X8, const double* eps, const double* mu, 
   return (int)cudaGetLastError();
 }
 
-template <typename T, int P, int Q>
-int mass_pq(const T* um, int64_t um_es, int64_t um_cs, const T* u0, int64_t u0_es, int64_t u0_cs, const T* Gw,
-            const T* eps, const T* mu, const CurvedTables& ct, int64_t ne, T* R, cudaStream_t s,
-            const int32_t* skip) {
-  constexpr int NQ3 = (P + 2) * (P + 2) * (P + 2);
-  const size_t sm = sizeof(T) * 12 * NQ3;
-  static std::atomic<uint64_t> configured_devices{0};
-  once_per_device(configured_devices, [&] {
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_mass_curved<T, P, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  });
-  // grid-stride over elements, one wave of co-resident CTAs (a skipped launch costs one wave)
-  static std::atomic<int> cap[64];
-  const int grid = wave_grid(k_mass_curved<T, P, Q>, 256, sm, ne, cap);
-  k_mass_curved<T, P, Q><<<grid, 256, sm, s>>>(um, um_es, um_cs, u0, u0_es, u0_cs, Gw, eps, mu, ctab<T>(ct), ne, R,
-                                                skip);
-  return (int)cudaGetLastError();
-}
-
-template <typename T>
-int launch_mass_curved(int P, int Q, const T* um, int64_t um_es, int64_t um_cs, const T* u0, int64_t u0_es,
-                       int64_t u0_cs, const T* Gw, const T* eps, const T* mu, const CurvedTables& ct, int64_t ne, T* R,
-                       cudaStream_t s, const int32_t* skip) {
-#define STM_MQ(p, q) \
-  if (P == p && Q == q) return mass_pq<T, p, q>(um, um_es, um_cs, u0, u0_es, u0_cs, Gw, eps, mu, ct, ne, R, s, skip);
-#define STM_MP(p) STM_MQ(p, 1) STM_MQ(p, 2) STM_MQ(p, 3) STM_MQ(p, 4) STM_MQ(p, 5) STM_MQ(p, 6)
-  STM_MP(0) STM_MP(1) STM_MP(2) STM_MP(3) STM_MP(4) STM_MP(5) STM_MP(6) STM_MP(7)
-#undef STM_MP
-#undef STM_MQ
-  return (int)cudaErrorInvalidValue;
-}
-
 template <typename S, typename X>
 void precond_curved(X* out, const S* V, int64_t ldv, int k, const double* y, const S* Pinv, int64_t qn3, int64_t ne,
                     bool add, cudaStream_t s, const int32_t* skip, const GmresState* st) {
@@ -353,12 +228,6 @@ int launch_energy_curved(int P, const double* u, const double* Gw, const double*
   return (int)cudaGetLastError();
 }
 
-template int launch_mass_curved<double>(int, int, const double*, int64_t, int64_t, const double*, int64_t, int64_t,
-                                        const double*, const double*, const double*, const CurvedTables&, int64_t,
-                                        double*, cudaStream_t, const int32_t*);
-template int launch_mass_curved<float>(int, int, const float*, int64_t, int64_t, const float*, int64_t, int64_t,
-                                       const float*, const float*, const float*, const CurvedTables&, int64_t, float*,
-                                       cudaStream_t, const int32_t*);
 template void precond_curved<double, double>(double*, const double*, int64_t, int, const double*, const double*,
                                              int64_t, int64_t, bool, cudaStream_t, const int32_t*, const GmresState*);
 template void precond_curved<float, float>(float*, const float*, int64_t, int, const double*, const float*, int64_t,

@@ -29,18 +29,11 @@ struct CurvedTables {
 int launch_metric(int P, const double* X8, const double* eps, const double* mu, int64_t ne, const CurvedTables& ct,
                   double* Gw, double* Pinv, int* bad, cudaStream_t s);
 
-// R[e][f][c][i][s] = mat_f (M_G (u_{i+1} - delta_{i0} u_0))[c][s] for every element.
+// R[e][f][c][i][s] = mat_f (M_G (u_{i+1} - delta_{i0} u_0))[c][s] for every element (curved_mass.cu).
 template <typename T>
 int launch_mass_curved(int P, int Q, const T* um, int64_t um_es, int64_t um_cs, const T* u0, int64_t u0_es,
                        int64_t u0_cs, const T* Gw, const T* eps, const T* mu, const CurvedTables& ct, int64_t ne, T* R,
                        cudaStream_t s, const int32_t* skip = nullptr);
-
-// The same FP32 mass term on the tensor cores (tcgen05.mma kind::tf32 with 3xTF32 split
-// products, accumulators in tensor memory) for 3 <= P <= 7; cudaErrorInvalidValue for other
-// degrees.  *err is set to 1 if a bounded wait of the kernel ran out (R is then incomplete).
-int launch_mass_curved_tc(int P, int Q, const float* um, int64_t um_es, int64_t um_cs, const float* u0, int64_t u0_es,
-                          int64_t u0_cs, const float* Gw, const float* eps, const float* mu, const CurvedTables& ct,
-                          int64_t ne, float* R, cudaStream_t s, const int32_t* skip, int* err);
 
 // z[e][f][c][i][s] = sum_d Pinv[e][f][c][d] v[e][f][d][i][s]   (add = false), or x += that (add = true);
 // with k > 0, v is the combination sum_{j<k} y[j] V[j] (ldv apart).

@@ -85,7 +85,7 @@ struct ApplyArgs {
   T* R = nullptr;                   // [ne][2][3][q][N3] residual (test layout)
   const int32_t* nbr = nullptr;     // [ne][6]
   const T* mass = nullptr;          // [ne][2][3]: eps G_c (E rows), mu G_c (H rows); nullptr: R already
-                                    //   holds the mass term (curved elements, written by k_mass_curved)
+                                    //   holds the mass term (curved elements, written by k_mass)
   int64_t n_elem = 0;
   Tables<T> tb{};
   // uneven (p, q): elements of one class are listed in elist; every per-element
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q), residual_min_block
           }
         }
       } else {
-        // curved elements: R already holds the mass term (k_mass_curved)
+        // curved elements: R already holds the mass term (k_mass)
         for (int it = threadIdx.x; it < NF * FB; it += blockDim.x) {
           const int fl = NF == 1 ? 0 : it / FB;
           const int w = it - fl * FB;
@@ -1080,7 +1080,7 @@ __host__ __device__ constexpr size_t fused_kry_smem(int P, int Q) {
 // Single-pass FP32 Krylov operator on uniform meshes (no slab-start mode, no load): the inner
 // operator of the mixed-precision solve.  MODE 0: A P^{-1} v on bricks (P^{-1} on load, the
 // mass term is v itself); MODE 1: A z on curved elements, the mass term already in R (the
-// tensor-core or CUDA-core curved mass, z = P^{-1} v from the 3x3 block pass); MODE 2: A z on
+// curved mass, z = P^{-1} v from the 3x3 block pass); MODE 2: A z on
 // general affine elements (constant 3x3 metric mass).  Same arithmetic as k_fused,
 // specialised:
 //  (a) forms y = sc B v and the mass term with no branches on the generic inputs;

@@ -273,7 +273,6 @@ struct stm_ctx {
   float* Pinv32 = nullptr;
   double* mass3_64 = nullptr;  // general affine elements: [ne][2][6] mat * G (constant metric)
   float* mass3_32 = nullptr;
-  int* tc_err = nullptr;       // trilinear meshes: set by the tensor-core mass kernel if a wait ran out
   int* wait_err = nullptr;     // set by the FP32 Krylov kernel if a bounded wait on its copies ran out
   double* el = nullptr;      // per-element energies (curved)
   CurvedTables ct{};
@@ -686,18 +685,9 @@ int apply(stm_ctx* c, double dt, const T* um, int um_layout, const T* u0, int u0
   }
   if (c->geometry == STM_GEOM_TRILINEAR) {
     // curved: the metric-dependent mass term goes first into R; the residual kernels add the rest
-    int em;
-    if constexpr (sizeof(T) == 4) {
-      if (!c->opts.no_tensor_cores && c->P >= 3 && c->tc_err)
-        em = launch_mass_curved_tc(c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, c->Gw32, c->eps32,
-                                   c->mu32, c->ct, c->ne, R, c->stream, skip, c->tc_err);
-      else
-        em = launch_mass_curved<T>(c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, curved_ptr<T>(c, 0),
-                                   curved_ptr<T>(c, 1), curved_ptr<T>(c, 2), c->ct, c->ne, R, c->stream, skip);
-    } else {
-      em = launch_mass_curved<T>(c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, curved_ptr<T>(c, 0),
-                                 curved_ptr<T>(c, 1), curved_ptr<T>(c, 2), c->ct, c->ne, R, c->stream, skip);
-    }
+    const int em =
+        launch_mass_curved<T>(c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, curved_ptr<T>(c, 0),
+                              curved_ptr<T>(c, 1), curved_ptr<T>(c, 2), c->ct, c->ne, R, c->stream, skip);
     c->launches += 1;
     if (em) return fail(c, STM_EDEVICE, std::string("curved mass launch: ") + cudaGetErrorString((cudaError_t)em));
     a.mass = nullptr;
@@ -1803,10 +1793,6 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
       int bad_h = 0;
       cudaMemcpy(&bad_h, bad_d, sizeof(int), cudaMemcpyDeviceToHost);
       cudaFree(bad_d);
-      if (!affine) {
-        ok = cudaMalloc(&c->tc_err, sizeof(int)) == cudaSuccess;
-        if (ok) cudaMemset(c->tc_err, 0, sizeof(int));
-      }
       if (affine) {
         std::vector<float> m3(c->h_mass3.begin(), c->h_mass3.end());
         ok = cudaMalloc(&c->mass3_64, c->h_mass3.size() * sizeof(double)) == cudaSuccess &&
@@ -1983,7 +1969,7 @@ int32_t stm_destroy(stm_ctx* c) {
                   c->x,       c->V32,     c->z32,    c->inv64, c->inv32, c->X8, c->eps64, c->mu64,
                   c->eps32,   c->mu32,    c->Gw64,   c->Gw32,  c->Pinv64, c->Pinv32, c->el, c->load64, c->load32,
                   c->sw64,    c->sw32,    c->kap64,  c->kap32, c->nkl,    c->tmat64, c->tmat32,
-                  c->mass3_64, c->mass3_32, c->tc_err, c->wait_err};
+                  c->mass3_64, c->mass3_32, c->wait_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -2482,12 +2468,6 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
       done = h.outer_done != 0;
       break;
     }
-  }
-  if (c->tc_err) {  // a bounded wait of the tensor-core mass kernel ran out: no valid result
-    int h_err = 0;
-    STM_CK(cudaMemcpyAsync(&h_err, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    STM_CK(cudaStreamSynchronize(c->stream));
-    if (h_err) return fail(c, STM_ETIMEOUT, "tensor-core mass kernel: a bounded wait ran out");
   }
   if (int rc = check_wait_err(c)) return rc;
   if (c->hp) extract_end_hp(c->state, c->x, c->off_test, c->off_state, c->pq, c->ne, c->stream);
