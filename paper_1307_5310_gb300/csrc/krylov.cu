@@ -79,21 +79,192 @@ struct Unroll {
   static constexpr int U = K <= 1 ? 4 : (K <= 3 ? 2 : 1);
 };
 
-template <typename S, int K>
-__global__ void __launch_bounds__(kRedThreads) k_multidot(const S* __restrict__ w, const S* __restrict__ V,
-                                                          int64_t ldv, int with_norm, int64_t n,
-                                                          double* __restrict__ partial, const int32_t* skip) {
-  if (skip && *skip) return;
+constexpr int kRedWarps = kRedThreads / 32;
+
+// Sums of the M per-thread values get(i) over the block in a fixed order (warp shuffles, then the
+// warp totals), written to partial[i * gridDim.x + blockIdx.x]: all values share one barrier.
+template <int M, typename F>
+__device__ __forceinline__ void block_partials(F&& get, double* __restrict__ partial) {
+  __shared__ double sh[M][kRedWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const double v = warp_sum(get(i));
+    if (lane == 0) sh[i][wid] = v;
+  }
+  __syncthreads();
+  for (int i = wid; i < M; i += kRedWarps) {
+    double v = lane < kRedWarps ? sh[i][lane] : 0.0;
+    v = warp_sum(v);
+    if (lane == 0) partial[(int64_t)i * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+// True in every thread of the block that is the last of the grid to arrive (its reads of the other
+// blocks' partial sums are then valid); the counter is back at 0 for the next launch.
+__device__ bool last_block(GmresState* st) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(&st->ticket, 1) == (int)gridDim.x - 1;
+    if (last) st->ticket = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// The grid's sums of m values in a fixed order (one warp per value: lane-strided, then a shuffle tree).
+__device__ void grid_sums(const double* __restrict__ partial, int m, double* out) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nb = gridDim.x;
+  for (int i = wid; i < m; i += kRedWarps) {
+    double v = 0.0;
+#pragma unroll 8
+    for (int b = lane; b < nb; b += 32) v += __ldcg(partial + (int64_t)i * nb + b);
+    v = warp_sum(v);
+    if (lane == 0) out[i] = v;
+  }
+  __syncthreads();
+}
+
+// ---- scalar steps of the device-side GMRES control, run by the last block of a reduction ----
+
+__device__ void outer_check(GmresState* st) {
+  st->k = 0;
+  st->skip_reo = 1;
+  const double beta = sqrt(st->red[0]);
+  const double ref = st->ref;
+  st->rel = ref > 0 ? beta / ref : beta;
+  if (!isfinite(st->rel)) {
+    st->status = -5;  // STM_ENAN
+    st->skip = 1;
+    st->halt = 1;
+    return;
+  }
+  bool done;
+  if (st->inexact) {
+    st->phi = sqrt(st->red[1]);
+    done = st->phi <= st->tol;
+  } else {
+    done = st->rel <= st->tol;
+  }
+  if (done) st->outer_done = 1;
+  st->skip = (done || st->iters >= st->max_it || beta == 0.0) ? 1 : 0;
+  st->halt = st->skip;
+}
+
+__device__ void cycle_init(GmresState* st, int slot_start, double floor_rel) {
+  if (st->skip) return;
+  const double b0 = sqrt(st->red[slot_start]);
+  if (!(b0 > 0.0)) {
+    st->skip = 1;
+    st->halt = 1;
+    return;
+  }
+  st->cycles += 1;
+  // v_0 = V[0] / alpha_0 with V[0] = R = -r: alpha_0 = -|start|
+  st->alpha[0] = -b0;
+  st->g[0] = b0;
+  const double target = st->inexact ? st->tol : st->tol * st->ref;
+  st->tol_abs = fmax(target, floor_rel * b0);
+}
+
+// Coefficients of one Gram-Schmidt pass over V[0..j] from the dot products v (whole block).
+__device__ void gs_step(GmresState* st, const double* v, int j, bool second) {
+  if ((int)threadIdx.x <= j) {
+    const int i = threadIdx.x;
+    const double ai = st->alpha[i], aj = st->alpha[j];
+    st->cc[i] = v[i] / (ai * ai);
+    const double h = v[i] / (ai * aj);
+    st->H[i * kMaxDots + j] = second ? st->H[i * kMaxDots + j] + h : h;
+  }
+}
+
+// Iteration j's Givens step from |W|^2 after the update; at the end of the cycle also the
+// triangular system and the combination coefficients (whole block, on a copy in shared memory).
+__device__ void givens_step(GmresState* st, double after, int j, int m) {
+  __shared__ double H[kMaxDots * kMaxDots], cs[kMaxDots], sn[kMaxDots], g[kMaxDots + 1], al[kMaxDots + 1];
+  __shared__ int stop;
+  __syncthreads();  // the column written by gs_step
+  const int t = threadIdx.x;
+  for (int k = t; k < kMaxDots * kMaxDots; k += blockDim.x) H[k] = st->H[k];
+  if (t < kMaxDots) {
+    cs[t] = st->cs[t];
+    sn[t] = st->sn[t];
+  }
+  if (t <= kMaxDots) {
+    g[t] = st->g[t];
+    al[t] = st->alpha[t];
+  }
+  __syncthreads();
+  if (t == 0) {
+    stop = 0;
+    if (!isfinite(after) || !isfinite(st->before)) {
+      st->status = -5;  // STM_ENAN
+      st->k = 0;
+      st->skip = 1;
+      st->halt = 1;
+      st->skip_reo = 1;
+    } else {
+      const double nw = sqrt(after);
+      const double aj = al[j];
+      st->alpha[j + 1] = aj < 0 ? -nw : nw;
+      double y0 = nw / fabs(aj);
+      double x0 = H[j];
+      for (int i = 0; i < j; ++i) {
+        const double x = x0, y = H[(i + 1) * kMaxDots + j];
+        H[i * kMaxDots + j] = cs[i] * x + sn[i] * y;
+        x0 = -sn[i] * x + cs[i] * y;
+      }
+      const double r = hypot(x0, y0);
+      const double c = r > 0 ? x0 / r : 1.0, s = r > 0 ? y0 / r : 0.0;
+      H[j * kMaxDots + j] = r;
+      const double g1 = -s * g[j];
+      g[j] = c * g[j];
+      g[j + 1] = g1;
+      st->cs[j] = c;
+      st->sn[j] = s;
+      st->g[j] = g[j];
+      st->g[j + 1] = g1;
+      st->iters += 1;
+      st->k = j + 1;
+      stop = fabs(g1) <= st->tol_abs || nw == 0.0 || st->iters >= st->max_it || j + 1 >= m;
+      if (stop) {
+        st->skip = 1;
+        st->skip_reo = 1;
+      }
+    }
+  }
+  __syncthreads();
+  if (t <= j) st->H[t * kMaxDots + j] = H[t * kMaxDots + j];
+  if (stop && t == 0) {
+    const int k = j + 1;
+    for (int i = k - 1; i >= 0; --i) {
+      double y = g[i];
+      for (int l = i + 1; l < k; ++l) y -= H[i * kMaxDots + l] * g[l];
+      g[i] = y / H[i * kMaxDots + i];
+    }
+    for (int i = 0; i < kMaxDots; ++i) st->yc[i] = i < k ? g[i] / al[i] : 0.0;
+    st->res = fabs(g[k]);
+  }
+}
+
+// Dot products of w with V[0..K-1] and |w|^2 (index K).  GS: the last block of the grid turns them
+// into iteration j = K - 1's Gram-Schmidt coefficients and Hessenberg column.
+template <typename S, int K, bool GS>
+__global__ void __launch_bounds__(kRedThreads) k_dots(const S* __restrict__ w, const S* __restrict__ V, int64_t ldv,
+                                                      int64_t n, double* __restrict__ partial, GmresState* st) {
+  if (GS && st->skip) return;
   using VT = typename Vec<S>::T;
   constexpr int W = Vec<S>::W, U = Unroll<K>::U;
-  __shared__ double sh[32];
   Acc<S> acc[K + 1];
   const int64_t nv = n / W;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   const VT* w4 = reinterpret_cast<const VT*>(w);
   int chunks = 0;
   for (int64_t c0 = tid; c0 < nv; c0 += nth * U) {
-    VT wv[U], vv[U][K > 0 ? K : 1];
+    VT wv[U], vv[U][K];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int64_t c = c0 + u * nth;
@@ -111,7 +282,7 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const S* __restrict__ 
           const S x = Vec<S>::get(wv[u], l);
 #pragma unroll
           for (int i = 0; i < K; ++i) acc[i].add(x, Vec<S>::get(vv[u][i], l));
-          if (with_norm) acc[K].add(x, x);
+          acc[K].add(x, x);
         }
         if ((++chunks & 3) == 0) {
 #pragma unroll
@@ -124,31 +295,47 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot(const S* __restrict__ 
     const S x = w[j];
 #pragma unroll
     for (int i = 0; i < K; ++i) acc[i].add(x, V[i * ldv + j]);
-    if (with_norm) acc[K].add(x, x);
+    acc[K].add(x, x);
   }
-#pragma unroll
-  for (int i = 0; i < K; ++i) {
-    const double r = block_sum(acc[i].get(), sh);
-    if (threadIdx.x == 0) partial[i * gridDim.x + blockIdx.x] = r;
-  }
-  if (with_norm) {
-    const double r = block_sum(acc[K].get(), sh);
-    if (threadIdx.x == 0) partial[K * gridDim.x + blockIdx.x] = r;
+  block_partials<K + 1>([&](int i) { return acc[i].get(); }, partial);
+  if constexpr (GS) {
+    if (!last_block(st)) return;
+    __shared__ double v[K + 1];
+    grid_sums(partial, K + 1, v);
+    gs_step(st, v, K - 1, false);
+    if (threadIdx.x == 0) st->before = v[K];
   }
 }
 
-template <typename S, int K>
-__global__ void __launch_bounds__(kRedThreads) k_axpy_norm(S* __restrict__ w, const S* __restrict__ V, int64_t ldv,
-                                                           Coef16 c, int64_t n, double* __restrict__ partial,
-                                                           const int32_t* skip, const double* cdev) {
-  if (skip && *skip) return;
+enum UpdateMode { kPlain, kOnly, kFirst, kSecond };
+
+// w -= sum_i c_i V[i] and |w|^2.  kPlain: c from the argument, partial sums only.  The others are the
+// update of iteration j = K - 1 with the coefficients of the device state: kOnly ends the iteration
+// (no second Gram-Schmidt pass); kFirst also forms the updated w's dot products with the same V chunks
+// (the second pass then needs no read of the basis for them) and its last block decides on that pass:
+// coefficients for it, or the end of the iteration; kSecond applies it and ends the iteration.  On the
+// 32^3 mixed solve both passes run in every iteration: a dot pass, two updates instead of two of each.
+template <typename S, int K, int MODE>
+__global__ void __launch_bounds__(kRedThreads) k_update(S* __restrict__ w, const S* __restrict__ V, int64_t ldv,
+                                                        Coef16 c, int64_t n, double* __restrict__ partial,
+                                                        GmresState* st, int m) {
+  if (MODE != kPlain && (MODE == kSecond ? st->skip_reo : st->skip)) return;
   using VT = typename Vec<S>::T;
-  constexpr int W = Vec<S>::W, U = Unroll<K>::U;
-  __shared__ double sh[32];
+  constexpr int W = Vec<S>::W, U = Unroll<K>::U, ND = MODE == kFirst ? K : 0;
   S cc[K > 0 ? K : 1];
+  if constexpr (sizeof(S) == 8 && K > 0) {
+    // one copy per lane: the compiler cannot make these uniform, and the FP64 pipe takes FMAs with
+    // three vector registers at full rate only
+    __shared__ double cl[K][32];
+    for (int k = threadIdx.x; k < K * 32; k += blockDim.x) cl[k / 32][k & 31] = MODE != kPlain ? st->cc[k / 32] : c.c[k / 32];
+    __syncthreads();
 #pragma unroll
-  for (int i = 0; i < K; ++i) cc[i] = (S)(cdev ? cdev[i] : c.c[i]);
-  Acc<S> acc;
+    for (int i = 0; i < K; ++i) cc[i] = cl[i][threadIdx.x & 31];
+  } else {
+#pragma unroll
+    for (int i = 0; i < K; ++i) cc[i] = (S)(MODE != kPlain ? st->cc[i] : c.c[i]);
+  }
+  Acc<S> acc, dot[ND > 0 ? ND : 1];
   const int64_t nv = n / W;
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   VT* w4 = reinterpret_cast<VT*>(w);
@@ -175,8 +362,14 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_norm(S* __restrict__ w, co
           for (int i = 0; i < K; ++i) x = fma(-cc[i], Vec<S>::get(vv[u][i], l), x);
           Vec<S>::set(wv[u], l, x);
           acc.add(x, x);
+#pragma unroll
+          for (int i = 0; i < ND; ++i) dot[i].add(x, Vec<S>::get(vv[u][i], l));
         }
-        if ((++chunks & 3) == 0) acc.flush();
+        if ((++chunks & 3) == 0) {
+          acc.flush();
+#pragma unroll
+          for (int i = 0; i < ND; ++i) dot[i].flush();
+        }
         if (K > 0) w4[cix] = wv[u];
       }
     }
@@ -187,9 +380,121 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_norm(S* __restrict__ w, co
     for (int i = 0; i < K; ++i) x = fma(-cc[i], V[i * ldv + j], x);
     if (K > 0) w[j] = x;
     acc.add(x, x);
+#pragma unroll
+    for (int i = 0; i < ND; ++i) dot[i].add(x, V[i * ldv + j]);
   }
-  const double r = block_sum(acc.get(), sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = r;
+  block_partials<ND + 1>([&](int i) { return i < ND ? dot[i].get() : acc.get(); }, partial);
+  if constexpr (MODE != kPlain) {
+    if (!last_block(st)) return;
+    __shared__ double v[ND + 1];
+    __shared__ int again;
+    grid_sums(partial, ND + 1, v);
+    const double after = v[ND];
+    if constexpr (MODE == kFirst) {
+      if (threadIdx.x == 0) {
+        again = after < 0.5 * st->before;  // the DGKS test
+        st->skip_reo = again ? 0 : 1;
+      }
+      __syncthreads();
+      if (again) {
+        gs_step(st, v, K - 1, true);
+        return;
+      }
+    }
+    if constexpr (MODE == kSecond) {
+      if (threadIdx.x == 0) st->skip_reo = 1;
+    }
+    givens_step(st, after, K - 1, m);
+  }
+}
+
+// |v|^2 of an FP64 vector, with the step that follows it in the slab solve (by the last block); CONV
+// also rounds the vector to float and takes |v32|^2.
+template <bool CONV>
+__global__ void __launch_bounds__(kRedThreads) k_norm_step(const double* __restrict__ v, float* __restrict__ v32,
+                                                           int64_t n, double* __restrict__ partial, GmresState* st,
+                                                           NormStep step) {
+  if (step.kind == NormStep::kSlabStart) {
+  } else if (CONV) {
+    if (st->skip) return;
+  } else if (st->halt) {
+    // the slab has stopped: this cycle applies nothing
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      st->k = 0;
+      st->skip = 1;
+      st->skip_reo = 1;
+    }
+    return;
+  }
+  const int64_t nv = n / 4;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+  const double2* v2 = reinterpret_cast<const double2*>(v);
+  Acc<double> acc;
+  Acc<float> acc32;
+  int chunks = 0;
+  for (int64_t c = tid; c < nv; c += nth) {  // four entries: two 16-byte loads
+    const double2 a = v2[2 * c], b = v2[2 * c + 1];
+    if constexpr (CONV) {
+      const float4 f = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+      reinterpret_cast<float4*>(v32)[c] = f;
+      acc32.add(f.x, f.x);
+      acc32.add(f.y, f.y);
+      acc32.add(f.z, f.z);
+      acc32.add(f.w, f.w);
+      if ((++chunks & 3) == 0) acc32.flush();
+    } else {
+      acc.add(a.x, a.x);
+      acc.add(a.y, a.y);
+      acc.add(b.x, b.x);
+      acc.add(b.y, b.y);
+    }
+  }
+  for (int64_t j = nv * 4 + tid; j < n; j += nth) {  // tail
+    if constexpr (CONV) {
+      const float f = (float)v[j];
+      v32[j] = f;
+      acc32.add(f, f);
+    } else {
+      acc.add(v[j], v[j]);
+    }
+  }
+  block_partials<1>([&](int) { return CONV ? acc32.get() : acc.get(); }, partial);
+  if (!last_block(st)) return;
+  __shared__ double sum[1];
+  grid_sums(partial, 1, sum);
+  if (threadIdx.x != 0) return;
+  switch (step.kind) {
+    case NormStep::kSlabStart:
+      st->red[0] = sum[0];
+      st->ref = sqrt(sum[0]);
+      st->tol = step.tol;
+      st->max_it = step.max_it;
+      st->inexact = step.inexact;
+      st->iters = 0;
+      st->cycles = 0;
+      st->status = 0;
+      st->outer_done = 0;
+      st->halt = 0;
+      st->skip = 0;
+      st->skip_reo = 1;
+      st->k = 0;
+      st->rel = 0.0;
+      st->phi = 0.0;
+      st->res = 0.0;
+      break;
+    case NormStep::kResidual:
+      st->red[0] = sum[0];
+      break;
+    case NormStep::kCheck:
+      st->red[step.slot] = sum[0];
+      outer_check(st);
+      if (step.init) cycle_init(st, step.slot, 0.0);
+      break;
+    case NormStep::kStart32:
+      st->red[2] = sum[0];
+      cycle_init(st, 2, 1e-6);
+      break;
+  }
 }
 
 __global__ void k_finish(const double* __restrict__ partial, int m, int nb, double* __restrict__ out) {
@@ -266,170 +571,6 @@ __global__ void k_convert(D* __restrict__ d, const S* __restrict__ s, int64_t n,
 }
 
 
-// ---- device-side GMRES control -------------------------------------------------------------
-// One block of kCtrlThreads threads: the fixed-order reduction of kRedBlocks partial sums per
-// value (warp i % warps sums value i lane-strided, then a shuffle tree), then thread 0 runs
-// the scalar logic of the restart cycle on the state in device memory.
-constexpr int kCtrlThreads = 512;
-
-__device__ void reduce_values(const double* __restrict__ partial, int m, double* out) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int i = wid; i < m; i += kCtrlThreads / 32) {
-    double v = 0.0;
-    for (int b = lane; b < kRedBlocks; b += 32) v += partial[i * kRedBlocks + b];
-    v = warp_sum(v);
-    if (lane == 0) out[i] = v;
-  }
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(kCtrlThreads) k_gm_reduce(const double* __restrict__ partial, GmresState* st,
-                                                             int slot, const int32_t* skip) {
-  if (skip && *skip) return;
-  __shared__ double v[1];
-  reduce_values(partial, 1, v);
-  if (threadIdx.x == 0) st->red[slot] = v[0];
-}
-
-__global__ void k_gm_slab_start(GmresState* st, double tol, int max_it, int inexact) {
-  st->ref = sqrt(st->red[0]);
-  st->tol = tol;
-  st->max_it = max_it;
-  st->inexact = inexact;
-  st->iters = 0;
-  st->cycles = 0;
-  st->status = 0;
-  st->outer_done = 0;
-  st->halt = 0;
-  st->skip = 0;
-  st->skip_reo = 1;
-  st->k = 0;
-  st->rel = 0.0;
-  st->phi = 0.0;
-  st->res = 0.0;
-}
-
-__global__ void k_gm_outer_check(GmresState* st) {
-  st->k = 0;
-  st->skip_reo = 1;
-  if (st->halt) {
-    st->skip = 1;
-    return;
-  }
-  const double beta = sqrt(st->red[0]);
-  const double ref = st->ref;
-  st->rel = ref > 0 ? beta / ref : beta;
-  if (!isfinite(st->rel)) {
-    st->status = -5;  // STM_ENAN
-    st->skip = 1;
-    st->halt = 1;
-    return;
-  }
-  bool done;
-  if (st->inexact) {
-    st->phi = sqrt(st->red[1]);
-    done = st->phi <= st->tol;
-  } else {
-    done = st->rel <= st->tol;
-  }
-  if (done) st->outer_done = 1;
-  st->skip = (done || st->iters >= st->max_it || beta == 0.0) ? 1 : 0;
-  st->halt = st->skip;
-}
-
-__global__ void k_gm_cycle_init(GmresState* st, int slot_start, double floor_rel) {
-  if (st->skip) return;
-  const double b0 = sqrt(st->red[slot_start]);
-  if (!(b0 > 0.0)) {
-    st->skip = 1;
-    st->halt = 1;
-    return;
-  }
-  st->cycles += 1;
-  // v_0 = V[0] / alpha_0 with V[0] = R = -r: alpha_0 = -|start|
-  st->alpha[0] = -b0;
-  st->g[0] = b0;
-  const double target = st->inexact ? st->tol : st->tol * st->ref;
-  st->tol_abs = fmax(target, floor_rel * b0);
-}
-
-__global__ void __launch_bounds__(kCtrlThreads) k_gm_gs(const double* __restrict__ partial, GmresState* st, int j,
-                                                         int second) {
-  if (second ? st->skip_reo : st->skip) return;
-  __shared__ double v[kMaxDots + 1];
-  reduce_values(partial, second ? j + 1 : j + 2, v);
-  if (threadIdx.x == 0) {
-    for (int i = 0; i <= j; ++i) {
-      st->cc[i] = v[i] / (st->alpha[i] * st->alpha[i]);
-      const double h = v[i] / (st->alpha[i] * st->alpha[j]);
-      st->H[i * kMaxDots + j] = second ? st->H[i * kMaxDots + j] + h : h;
-    }
-    if (!second) st->before = v[j + 1];
-  }
-}
-
-__global__ void __launch_bounds__(kCtrlThreads) k_gm_after(const double* __restrict__ partial, GmresState* st,
-                                                            int reorth) {
-  if (st->skip) {
-    st->skip_reo = 1;
-    return;
-  }
-  __shared__ double v[1];
-  reduce_values(partial, 1, v);
-  if (threadIdx.x == 0) {
-    st->after = v[0];
-    st->skip_reo = (reorth && v[0] < 0.5 * st->before) ? 0 : 1;
-  }
-}
-
-__global__ void __launch_bounds__(kCtrlThreads) k_gm_givens(const double* __restrict__ partial, GmresState* st, int j,
-                                                             int m, int reo_mode) {
-  if (st->skip) return;
-  __shared__ double v[1];
-  const bool fresh = reo_mode ? !st->skip_reo : true;  // uniform over the block
-  if (fresh) reduce_values(partial, 1, v);
-  if (threadIdx.x != 0) return;
-  const double after = fresh ? v[0] : st->after;
-  double* H = st->H;
-  if (!isfinite(after) || !isfinite(st->before)) {
-    st->status = -5;  // STM_ENAN
-    st->skip = 1;
-    st->halt = 1;
-    return;
-  }
-  const double nw = sqrt(after);
-  st->alpha[j + 1] = st->alpha[j] < 0 ? -nw : nw;
-  H[(j + 1) * kMaxDots + j] = nw / fabs(st->alpha[j]);
-  for (int i = 0; i < j; ++i) {
-    const double x = H[i * kMaxDots + j], y = H[(i + 1) * kMaxDots + j];
-    H[i * kMaxDots + j] = st->cs[i] * x + st->sn[i] * y;
-    H[(i + 1) * kMaxDots + j] = -st->sn[i] * x + st->cs[i] * y;
-  }
-  const double x = H[j * kMaxDots + j], y = H[(j + 1) * kMaxDots + j];
-  const double r = hypot(x, y);
-  st->cs[j] = r > 0 ? x / r : 1.0;
-  st->sn[j] = r > 0 ? y / r : 0.0;
-  H[j * kMaxDots + j] = r;
-  H[(j + 1) * kMaxDots + j] = 0.0;
-  st->g[j + 1] = -st->sn[j] * st->g[j];
-  st->g[j] = st->cs[j] * st->g[j];
-  st->iters += 1;
-  st->k = j + 1;
-  if (fabs(st->g[j + 1]) <= st->tol_abs || nw == 0.0 || st->iters >= st->max_it || j + 1 >= m) st->skip = 1;
-}
-
-__global__ void k_gm_backsub(GmresState* st) {
-  const int k = st->k;
-  double y[kMaxDots];
-  for (int i = k - 1; i >= 0; --i) {
-    double t = st->g[i];
-    for (int l = i + 1; l < k; ++l) t -= st->H[i * kMaxDots + l] * y[l];
-    y[i] = t / st->H[i * kMaxDots + i];
-  }
-  for (int i = 0; i < kMaxDots; ++i) st->yc[i] = i < k ? y[i] / st->alpha[i] : 0.0;
-  st->res = fabs(st->g[k]);
-}
-
 inline int grid_for(int64_t n) {
   int64_t g = (n + kRedThreads - 1) / kRedThreads;
   return (int)(g < 4 * kRedBlocks ? (g < 1 ? 1 : g) : 4 * kRedBlocks);
@@ -437,16 +578,10 @@ inline int grid_for(int64_t n) {
 
 inline bool small(int64_t n) { return n <= (int64_t)0xffffffffLL; }
 
-template <typename S, int K>
-void multidot_k(const S* w, const S* V, int64_t ldv, bool with_norm, int64_t n, double* partial, cudaStream_t s,
-                const int32_t* skip) {
-  k_multidot<S, K><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, with_norm ? 1 : 0, n, partial, skip);
-}
-
-template <typename S, int K>
-void axpy_k(S* w, const S* V, int64_t ldv, const Coef16& c, int64_t n, double* partial, cudaStream_t s,
-            const int32_t* skip, const double* cdev) {
-  k_axpy_norm<S, K><<<kRedBlocks, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, skip, cdev);
+// Blocks of a reduction over nv vectors: one vector a thread on small problems, at most kRedBlocks.
+inline int red_grid(int64_t nv) {
+  const int64_t g = (nv + kRedThreads - 1) / kRedThreads;
+  return (int)(g < 1 ? 1 : (g < kRedBlocks ? g : kRedBlocks));
 }
 
 template <typename S, typename X, int K>
@@ -458,7 +593,6 @@ void combine_k(X* x, const S* V, int64_t ldv, const Coef16& y, const S* inv, int
 
 #define STM_SWITCH_K(k, CALL)  \
   switch (k) {                 \
-    case 0: CALL(0); break;    \
     case 1: CALL(1); break;    \
     case 2: CALL(2); break;    \
     case 3: CALL(3); break;    \
@@ -478,22 +612,57 @@ void combine_k(X* x, const S* V, int64_t ldv, const Coef16& y, const S* inv, int
 
 }  // namespace
 
-template <typename S>
-void multidot(const S* w, const S* V, int64_t ldv, int k, bool with_norm, int64_t n, double* partial, double* out,
-              cudaStream_t s, const int32_t* skip) {
-#define STM_MD(K) multidot_k<S, K>(w, V, ldv, with_norm, n, partial, s, skip)
-  STM_SWITCH_K(k, STM_MD)
-#undef STM_MD
-  if (out) k_finish<<<1, 512, 0, s>>>(partial, k + (with_norm ? 1 : 0), kRedBlocks, out);
+void dot(const double* w, const double* v, int64_t n, double* partial, double* out, cudaStream_t s) {
+  const int g = red_grid(n / Vec<double>::W);
+  k_dots<double, 1, false><<<g, kRedThreads, 0, s>>>(w, v, 0, n, partial, nullptr);
+  k_finish<<<1, 32, 0, s>>>(partial, 1, g, out);
+}
+
+void axpy_norm(double* w, const double* v, double c, int64_t n, double* partial, double* out, cudaStream_t s) {
+  const int g = red_grid(n / Vec<double>::W);
+  Coef16 cc{};
+  cc.c[0] = c;
+  if (v) k_update<double, 1, kPlain><<<g, kRedThreads, 0, s>>>(w, v, 0, cc, n, partial, nullptr, 0);
+  else k_update<double, 0, kPlain><<<g, kRedThreads, 0, s>>>(w, w, 0, cc, n, partial, nullptr, 0);
+  k_finish<<<1, 32, 0, s>>>(partial, 1, g, out);
 }
 
 template <typename S>
-void axpy_norm(S* w, const S* V, int64_t ldv, int k, const Coef16& c, int64_t n, double* partial, double* out,
-               cudaStream_t s, const int32_t* skip, const double* cdev) {
-#define STM_AX(K) axpy_k<S, K>(w, V, ldv, c, n, partial, s, skip, cdev)
-  STM_SWITCH_K(k, STM_AX)
-#undef STM_AX
-  if (out) k_finish<<<1, 32, 0, s>>>(partial, 1, kRedBlocks, out);
+void gmres_dots(const S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st,
+                cudaStream_t s) {
+  const int g = red_grid(n / Vec<S>::W);
+#define STM_MD(K) k_dots<S, K, true><<<g, kRedThreads, 0, s>>>(w, V, ldv, n, partial, st)
+  STM_SWITCH_K(j + 1, STM_MD)
+#undef STM_MD
+}
+
+template <typename S>
+void gmres_update(S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st, int m, bool reorth,
+                  cudaStream_t s) {
+  const int g = red_grid(n / Vec<S>::W);
+  const Coef16 c{};
+#define STM_UP(K) k_update<S, K, kOnly><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
+#define STM_UP1(K) k_update<S, K, kFirst><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
+#define STM_UP2(K) k_update<S, K, kSecond><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
+  if (reorth) {
+    STM_SWITCH_K(j + 1, STM_UP1)
+    STM_SWITCH_K(j + 1, STM_UP2)
+  } else {
+    STM_SWITCH_K(j + 1, STM_UP)
+  }
+#undef STM_UP
+#undef STM_UP1
+#undef STM_UP2
+}
+
+void gmres_norm(const double* v, int64_t n, double* partial, GmresState* st, const NormStep& step, cudaStream_t s) {
+  k_norm_step<false><<<red_grid(n / 4), kRedThreads, 0, s>>>(v, nullptr, n, partial, st, step);
+}
+
+void gmres_start32(const double* v, float* v32, int64_t n, double* partial, GmresState* st, cudaStream_t s) {
+  NormStep step{};
+  step.kind = NormStep::kStart32;
+  k_norm_step<true><<<red_grid(n / 4), kRedThreads, 0, s>>>(v, v32, n, partial, st, step);
 }
 
 template <typename S>
@@ -523,38 +692,12 @@ void convert(D* dst, const S* src, int64_t n, cudaStream_t s, const int32_t* ski
 }
 
 
-void gmres_reduce(const double* partial, GmresState* st, int slot, cudaStream_t s, const int32_t* skip) {
-  k_gm_reduce<<<1, kCtrlThreads, 0, s>>>(partial, st, slot, skip);
-}
-void gmres_slab_start(GmresState* st, double tol, int max_it, int inexact, cudaStream_t s) {
-  k_gm_slab_start<<<1, 1, 0, s>>>(st, tol, max_it, inexact);
-}
-void gmres_outer_check(GmresState* st, cudaStream_t s) { k_gm_outer_check<<<1, 1, 0, s>>>(st); }
-void gmres_cycle_init(GmresState* st, int slot_start, double floor_rel, cudaStream_t s) {
-  k_gm_cycle_init<<<1, 1, 0, s>>>(st, slot_start, floor_rel);
-}
-void gmres_gs(const double* partial, GmresState* st, int j, int second, cudaStream_t s) {
-  k_gm_gs<<<1, kCtrlThreads, 0, s>>>(partial, st, j, second);
-}
-void gmres_after(const double* partial, GmresState* st, int reorth, cudaStream_t s) {
-  k_gm_after<<<1, kCtrlThreads, 0, s>>>(partial, st, reorth);
-}
-void gmres_givens(const double* partial, GmresState* st, int j, int m, int reo_mode, cudaStream_t s) {
-  k_gm_givens<<<1, kCtrlThreads, 0, s>>>(partial, st, j, m, reo_mode);
-}
-void gmres_backsub(GmresState* st, int m, cudaStream_t s) {
-  (void)m;
-  k_gm_backsub<<<1, 1, 0, s>>>(st);
-}
-
-template void multidot<double>(const double*, const double*, int64_t, int, bool, int64_t, double*, double*,
-                               cudaStream_t, const int32_t*);
-template void multidot<float>(const float*, const float*, int64_t, int, bool, int64_t, double*, double*,
-                              cudaStream_t, const int32_t*);
-template void axpy_norm<double>(double*, const double*, int64_t, int, const Coef16&, int64_t, double*, double*,
-                                cudaStream_t, const int32_t*, const double*);
-template void axpy_norm<float>(float*, const float*, int64_t, int, const Coef16&, int64_t, double*, double*,
-                               cudaStream_t, const int32_t*, const double*);
+template void gmres_dots<double>(const double*, const double*, int64_t, int, int64_t, double*, GmresState*, cudaStream_t);
+template void gmres_dots<float>(const float*, const float*, int64_t, int, int64_t, double*, GmresState*, cudaStream_t);
+template void gmres_update<double>(double*, const double*, int64_t, int, int64_t, double*, GmresState*, int, bool,
+                                   cudaStream_t);
+template void gmres_update<float>(float*, const float*, int64_t, int, int64_t, double*, GmresState*, int, bool,
+                                  cudaStream_t);
 template void precond_apply<double>(double*, const double*, const double*, int64_t, int64_t, cudaStream_t,
                                     const int32_t*);
 template void precond_apply<float>(float*, const float*, const float*, int64_t, int64_t, cudaStream_t,

@@ -5,6 +5,12 @@
 // FP64.  With S = float (the inner solve of the mixed-precision path) each
 // thread sums products of 8 consecutive entries in FP32 and accumulates those
 // partial sums in FP64; the grid and block reductions are FP64.
+//
+// The last block of a reduction to arrive sums the grid's partials and takes the scalar step that
+// needs them (Gram-Schmidt coefficients, Givens rotation, stop tests, triangular solve), so an
+// iteration is two launches besides the operator (three with a second Gram-Schmidt pass) instead of
+// four (eight) and no single-thread kernel walks the state in device memory.  4^3 elements, p = 2,
+// q = 1, FP64 to 1e-12 (26 iterations, both passes): 2.12 -> 1.15 ms per slab.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -44,22 +50,18 @@ struct GmresState {
   int32_t outer_done;             // 1: the slab's stop test holds
   int32_t inexact;                // 1: stop on the weighted norm (eta_it), 0: on rel
   int32_t cycles;                 // restart cycles started
+  int32_t ticket;                 // blocks of the running reduction that have arrived (0 between launches)
   int32_t halt;                   // 1: the slab solve has stopped (stop test, cap, zero residual or
                                   //    error); every later kernel of the slab is skipped
 };
 
-// out[i] = sum_n w[n] V[i*ldv + n] for i < k (k <= 15), and out[k] = sum_n w[n]^2
-// if with_norm.  partial: (k+1) * kRedBlocks doubles of scratch.  out == nullptr:
-// only the partial sums are written (a control kernel reduces them).
-template <typename S>
-void multidot(const S* w, const S* V, int64_t ldv, int k, bool with_norm, int64_t n, double* partial, double* out,
-              cudaStream_t s, const int32_t* skip = nullptr);
+// partial: kMaxDots * kRedBlocks doubles of scratch for every reduction below.
 
-// w[n] -= sum_{i<k} c[i] V[i*ldv + n] (k may be 0), then out[0] = sum_n w[n]^2.  With
-// cdev non-null the coefficients are read from device memory instead of c.
-template <typename S>
-void axpy_norm(S* w, const S* V, int64_t ldv, int k, const Coef16& c, int64_t n, double* partial, double* out,
-               cudaStream_t s, const int32_t* skip = nullptr, const double* cdev = nullptr);
+// out[0] = sum_n w[n] v[n].
+void dot(const double* w, const double* v, int64_t n, double* partial, double* out, cudaStream_t s);
+
+// w[n] -= c v[n] (v null: w unchanged), then out[0] = sum_n w[n]^2.
+void axpy_norm(double* w, const double* v, double c, int64_t n, double* partial, double* out, cudaStream_t s);
 
 // z[n] = v[n] * inv[n / blk]  (blk = entries per (element, field, component) block).
 template <typename S>
@@ -72,28 +74,35 @@ template <typename S, typename X>
 void precond_combine(X* x, const S* V, int64_t ldv, int k, const Coef16& y, const S* inv, int64_t blk, int64_t n,
                      cudaStream_t s, const GmresState* st = nullptr);
 
-// ---- device-side GMRES control (one block each; partial: kRedBlocks sums per value) ----
-// st->red[slot] = sum of the partials of one reduction (fixed order).
-void gmres_reduce(const double* partial, GmresState* st, int slot, cudaStream_t s, const int32_t* skip = nullptr);
-// Slab start: st->ref = sqrt(red[0]); iteration count, flags and targets reset.
-void gmres_slab_start(GmresState* st, double tol, int max_it, int inexact, cudaStream_t s);
-// The slab's stop test on the true residual (norm^2 in red[0], weighted norm^2 in red[1]
-// if inexact, R6): sets outer_done, and skip when done, at the iteration cap or at R = 0.
-void gmres_outer_check(GmresState* st, cudaStream_t s);
-// Restart-cycle start (unless skipped): v_0 = start / (-|start|) with |start|^2 from
-// red[slot_start], and the cycle threshold max(target, floor_rel |start|).
-void gmres_cycle_init(GmresState* st, int slot_start, double floor_rel, cudaStream_t s);
-// Iteration j, after the multi-dot of W with V[0..j] (+ |W|^2): H column and the
-// Gram-Schmidt coefficients (second = 1: the DGKS pass, added to the column).
-void gmres_gs(const double* partial, GmresState* st, int j, int second, cudaStream_t s);
-// After the update's norm: with reorth, record |W|^2 and decide on a second pass.
-void gmres_after(const double* partial, GmresState* st, int reorth, cudaStream_t s);
-// Iteration j's Givens step; stops the cycle on |g_{j+1}| <= tol_abs, breakdown, the
-// iteration cap or the end of the cycle (j = m - 1).  reo_mode = 1: |W|^2 comes from the
-// second pass's partials when that pass ran, else from st->after.
-void gmres_givens(const double* partial, GmresState* st, int j, int m, int reo_mode, cudaStream_t s);
-// End of the cycle: y from the triangular system, yc = y / alpha.
-void gmres_backsub(GmresState* st, int m, cudaStream_t s);
+// ---- device-side GMRES: reductions whose last block takes the scalar step that follows ----
+// Each launch is skipped on the device once the cycle (st->skip) or the slab (st->halt) has stopped.
+
+// The step after the norm of an FP64 vector.
+struct NormStep {
+  enum Kind {
+    kSlabStart,  // st->ref = norm; iteration count, flags and targets reset (tol, max_it, inexact)
+    kResidual,   // red[0] = norm^2 (inexact solve: the weighted norm follows)
+    kCheck,      // red[slot] = norm^2, the slab's stop test on the true residual (R6): sets
+                 // outer_done, and skip when done, at the iteration cap or at R = 0; then, with
+                 // init, the start of the restart cycle: v_0 = start / (-|start|) and its threshold
+    kStart32     // red[2] = |v32|^2 and the start of an FP32 cycle (threshold at least 1e-6 |start|)
+  } kind = kResidual;
+  double tol = 0.0;
+  int max_it = 0, inexact = 0, slot = 0, init = 0;
+};
+void gmres_norm(const double* v, int64_t n, double* partial, GmresState* st, const NormStep& step, cudaStream_t s);
+// v32 = (float) v, then the kStart32 step.
+void gmres_start32(const double* v, float* v32, int64_t n, double* partial, GmresState* st, cudaStream_t s);
+// Iteration j: dot products of w with V[0..j] and |w|^2, the Gram-Schmidt coefficients and H column.
+template <typename S>
+void gmres_dots(const S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st,
+                cudaStream_t s);
+// Iteration j: w -= sum_i cc[i] V[i] and |w|^2; with reorth a second pass where |w| fell below 1/sqrt(2)
+// of its value (the DGKS test); then the Givens step, which stops the cycle on |g_{j+1}| <= tol_abs,
+// breakdown, the iteration cap or its end (j = m - 1) and there solves for the coefficients yc.
+template <typename S>
+void gmres_update(S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st, int m, bool reorth,
+                  cudaStream_t s);
 
 // out = 1/2 sum_n mass[n / n3] u[n]^2 (state layout, blocks of n3 per (element, field, component)).
 void energy_brick(const double* u, const double* mass, int64_t n3, int64_t n, double* partial, double* out,

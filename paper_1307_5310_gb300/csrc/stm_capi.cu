@@ -1196,25 +1196,6 @@ __global__ void k_extract_end(double* state, const double* x, int64_t q, int64_t
 
 int grid1(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 4096); }
 
-// ||v||^2 (fixed-order reduction, FP64 accumulation).
-template <typename S>
-int norm2(stm_ctx* c, S* v, int64_t n, double* out) {
-  axpy_norm<S>(v, v, 0, 0, Coef16{}, n, c->red_partial, c->red_out, c->stream);
-  c->launches += 2;
-  STM_CK(cudaMemcpyAsync(c->h_pinned, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  STM_CK(cudaStreamSynchronize(c->stream));
-  *out = c->h_pinned[0];
-  return STM_OK;
-}
-
-// One restart cycle of right-preconditioned GMRES on the unknowns (Sec. 5.4),
-// with the basis kept unnormalised: v_i = V_i / alpha_i (alpha_i signed).
-// On entry V[0] holds the start vector with v_0 = V[0] / a0 the normalised
-// residual r / |r|, |a0| = |r|.  Classical Gram-Schmidt (one fused dot pass,
-// one fused update + norm pass), with an optional second pass when the norm
-// drops below 1/sqrt(2) of its value before the update.  Returns the number k
-// of basis vectors used and the coefficients yc[i] such that the correction
-// is P^{-1} sum_{i<k} yc[i] V[i]; *res is the residual norm estimate |g_k|.
 // Weights of the iteration-error bound of Sec. 5.3 (Eq. a_posteriori:iteration):
 // eta_it^2 = 4 sum_n [(2 t_N/eps_min + dt^2/(2 t_N eps_min)) |R_E|^2_{W'} + (same, mu) |R_H|^2_{W'}],
 // with the dual norm on the test space |R|^2_{W'} = R^T M_W^{-1} R and, on
@@ -1294,24 +1275,11 @@ int gmres_iterations(stm_ctx* c, double dt, S* V, int64_t ldv, S* z, int64_t n) 
       if ((rc = linop_pre<S>(c, dt, Vj, W, skip))) return rc;
     }
     if (c->opts.eta_tol > 0) scale_blocks<S>(c, W, sw_ptr<S>(c), n, skip);  // residual space weighted by S
-    multidot<S>(W, V, ldv, j + 1, true, n, c->red_partial, nullptr, c->stream, skip);
-    gmres_gs(c->red_partial, st, j, 0, c->stream);
-    axpy_norm<S>(W, V, ldv, j + 1, Coef16{}, n, c->red_partial, nullptr, c->stream, skip, st->cc);
-    c->launches += 4;
-    if (c->opts.reorth) {
-      const int32_t* skip2 = &st->skip_reo;
-      gmres_after(c->red_partial, st, 1, c->stream);
-      multidot<S>(W, V, ldv, j + 1, false, n, c->red_partial, nullptr, c->stream, skip2);
-      gmres_gs(c->red_partial, st, j, 1, c->stream);
-      axpy_norm<S>(W, V, ldv, j + 1, Coef16{}, n, c->red_partial, nullptr, c->stream, skip2, st->cc);
-      c->launches += 4;
-    }
-    gmres_givens(c->red_partial, st, j, m, c->opts.reorth ? 1 : 0, c->stream);
-    c->launches += 1;
+    gmres_dots<S>(W, V, ldv, j, n, c->red_partial, st, c->stream);
+    gmres_update<S>(W, V, ldv, j, n, c->red_partial, st, m, c->opts.reorth != 0, c->stream);
+    c->launches += c->opts.reorth ? 3 : 2;
   }
   c->it_marks[m] = c->timed.size();
-  gmres_backsub(st, m, c->stream);
-  c->launches += 1;
   STM_CK(cudaGetLastError());
   return STM_OK;
 }
@@ -1346,21 +1314,20 @@ int launch_cycle(stm_ctx* c, double dt, const double* b, bool mixed, int64_t ldv
   // once the slab has stopped (st->halt), this cycle's kernels are all no-ops
   const int32_t* halt = &st->halt;
   if ((rc = resid64(c, dt, c->x, b, R64, halt))) return rc;
-  axpy_norm<double>(R64, R64, 0, 0, Coef16{}, n, c->red_partial, nullptr, c->stream, halt);
-  gmres_reduce(c->red_partial, st, 0, c->stream, halt);
-  c->launches += 2;
+  // V[0] = R = -r, so v_0 = V[0] / (-beta) of an FP64 cycle starts with the stop test
+  NormStep step{};
   if (inexact) {  // GMRES then works on the weighted residual S R
+    step.kind = NormStep::kResidual;
+    gmres_norm(R64, n, c->red_partial, st, step, c->stream);
     scale_blocks<double>(c, R64, c->sw64, n, halt);
-    axpy_norm<double>(R64, R64, 0, 0, Coef16{}, n, c->red_partial, nullptr, c->stream, halt);
-    gmres_reduce(c->red_partial, st, 1, c->stream, halt);
-    c->launches += 2;
+    c->launches += 1;
   }
-  gmres_outer_check(st, c->stream);
+  step.kind = NormStep::kCheck;
+  step.slot = inexact ? 1 : 0;
+  step.init = mixed ? 0 : 1;
+  gmres_norm(R64, n, c->red_partial, st, step, c->stream);
   c->launches += 1;
   if (!mixed) {
-    // V[0] = R = -r, so v_0 = V[0] / (-beta)
-    gmres_cycle_init(st, inexact ? 1 : 0, 0.0, c->stream);
-    c->launches += 1;
     if ((rc = gmres_iterations<double>(c, dt, c->V, ldv, c->z, n))) return rc;
     if (curved) precond_curved<double, double>(c->x, c->V, ldv, 0, nullptr, c->Pinv64, qn3, c->ne, true, c->stream,
                                                nullptr, st);
@@ -1370,11 +1337,8 @@ int launch_cycle(stm_ctx* c, double dt, const double* b, bool mixed, int64_t ldv
   } else {
     // FP32 inner GMRES(m) cycle on A d = r, started from the rounded FP64 residual; the inner
     // target is the outer one or what FP32 can resolve (1e-6 of the start), whichever is larger
-    convert<float, double>(c->V32, R64, n, c->stream, &st->skip);
-    axpy_norm<float>(c->V32, c->V32, 0, 0, Coef16{}, n, c->red_partial, nullptr, c->stream, &st->skip);
-    gmres_reduce(c->red_partial, st, 2, c->stream, &st->skip);
-    gmres_cycle_init(st, 2, 1e-6, c->stream);
-    c->launches += 4;
+    gmres_start32(R64, c->V32, n, c->red_partial, st, c->stream);
+    c->launches += 1;
     if ((rc = gmres_iterations<float>(c, dt, c->V32, ldv, c->z32, n))) return rc;
     if (curved) precond_curved<float, double>(c->x, c->V32, ldv, 0, nullptr, c->Pinv32, qn3, c->ne, true, c->stream,
                                               nullptr, st);
@@ -2217,7 +2181,7 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
   }
   double *x = buf, *r = buf + n, *pv = buf + 2 * n, *Ap = buf + 3 * n, *z = buf + 4 * n, *bd = buf + 5 * n;
   auto dot = [&](const double* a, const double* b, double* out) -> int {
-    multidot<double>(a, b, 0, 1, false, n, c->red_partial, c->red_out, c->stream);
+    stm::dot(a, b, n, c->red_partial, c->red_out, c->stream);
     c->launches += 2;
     STM_CK(cudaMemcpyAsync(c->h_pinned, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     STM_CK(cudaStreamSynchronize(c->stream));
@@ -2244,9 +2208,7 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
       if (restart > 0) {  // true residual r = b - M x
         if ((rc = mass(x, Ap))) break;
         STM_CK(cudaMemcpyAsync(r, bd, n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-        Coef16 cm{};
-        cm.c[0] = 1.0;
-        axpy_norm<double>(r, Ap, 0, 1, cm, n, c->red_partial, c->red_out, c->stream);
+        axpy_norm(r, Ap, 1.0, n, c->red_partial, c->red_out, c->stream);
         c->launches += 2;
         STM_CK(cudaMemcpyAsync(c->h_pinned, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         STM_CK(cudaStreamSynchronize(c->stream));
@@ -2261,11 +2223,8 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
         double pAp;
         if ((rc = dot(pv, Ap, &pAp))) break;
         const double alpha = rz / pAp;
-        Coef16 ca{}, cr{};
-        ca.c[0] = -alpha;
-        cr.c[0] = alpha;
-        axpy_norm<double>(x, pv, 0, 1, ca, n, c->red_partial, c->red_out, c->stream);  // x += alpha p
-        axpy_norm<double>(r, Ap, 0, 1, cr, n, c->red_partial, c->red_out, c->stream);  // r -= alpha Ap
+        axpy_norm(x, pv, -alpha, n, c->red_partial, c->red_out, c->stream);  // x += alpha p
+        axpy_norm(r, Ap, alpha, n, c->red_partial, c->red_out, c->stream);   // r -= alpha Ap
         c->launches += 4;
         STM_CK(cudaMemcpyAsync(c->h_pinned, c->red_out, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         STM_CK(cudaStreamSynchronize(c->stream));
@@ -2274,10 +2233,8 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
         c->launches += 1;
         double rz1;
         if ((rc = dot(r, z, &rz1))) break;
-        Coef16 cb{};
-        cb.c[0] = -rz1 / rz;
+        axpy_norm(z, pv, -rz1 / rz, n, c->red_partial, c->red_out, c->stream);  // z += beta p
         rz = rz1;
-        axpy_norm<double>(z, pv, 0, 1, cb, n, c->red_partial, c->red_out, c->stream);  // z += beta p
         c->launches += 2;
         std::swap(pv, z);
       }
@@ -2436,10 +2393,13 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
   // reference: ||R(U^(0))|| with all unknowns zero (R6), kept on the device
   STM_CK(cudaMemsetAsync(c->x, 0, n * sizeof(double), c->stream));
   if ((rc = resid64(c, dt, c->x, b, c->z))) return rc;
-  axpy_norm<double>(c->z, c->z, 0, 0, Coef16{}, n, c->red_partial, nullptr, c->stream);
-  gmres_reduce(c->red_partial, st, 0, c->stream);
-  gmres_slab_start(st, target, c->opts.max_it, inexact ? 1 : 0, c->stream);
-  c->launches += 3;
+  NormStep start{};
+  start.kind = NormStep::kSlabStart;
+  start.tol = target;
+  start.max_it = c->opts.max_it;
+  start.inexact = inexact ? 1 : 0;
+  gmres_norm(c->z, n, c->red_partial, st, start, c->stream);
+  c->launches += 1;
   // initial guess: u_1 = u_0, higher modes 0 (or all unknowns 0: x is already zero)
   if (!c->opts.zero_guess) {
     if (c->hp) init_guess_hp(c->x, c->state, c->off_test, c->off_state, c->pq, c->ne, c->stream);
