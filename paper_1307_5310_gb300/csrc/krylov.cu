@@ -1,5 +1,9 @@
 #include "krylov.cuh"
 
+#include <atomic>
+
+#include "residual.cuh"
+
 namespace stm {
 
 namespace {
@@ -81,22 +85,43 @@ struct Unroll {
 
 constexpr int kRedWarps = kRedThreads / 32;
 
-// Sums of the M per-thread values get(i) over the block in a fixed order (warp shuffles, then the
-// warp totals), written to partial[i * gridDim.x + blockIdx.x]: all values share one barrier.
+constexpr int log2_ceil(int m) { return m <= 1 ? 0 : 1 + log2_ceil((m + 1) / 2); }
+
+// Sums of the M per-thread values get(i) over the block in a fixed order, written to
+// partial[i * gridDim.x + blockIdx.x].  Within a warp the values are halved between lane halves at
+// each exchange (about M additions a lane instead of 5 M: on small problems these sums are what the
+// FP64 pipe does), then the warp totals in groups of eight lanes.
 template <int M, typename F>
 __device__ __forceinline__ void block_partials(F&& get, double* __restrict__ partial) {
-  __shared__ double sh[M][kRedWarps];
+  constexpr int LG = log2_ceil(M), MP = 1 << LG;
+  static_assert(M <= 32 && kRedWarps == 8, "one value per lane, eight warps");
+  __shared__ double sh[MP][kRedWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double v[MP];
 #pragma unroll
-  for (int i = 0; i < M; ++i) {
-    const double v = warp_sum(get(i));
-    if (lane == 0) sh[i][wid] = v;
+  for (int i = 0; i < MP; ++i) v[i] = i < M ? get(i) : 0.0;
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, cnt = MP >> st;
+    if (cnt > 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < cnt / 2; ++i) {
+        const double send = up ? v[i] : v[i + cnt / 2], keep = up ? v[i + cnt / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
   }
+  // lane l holds the total of value l >> (5 - LG)
+  if ((lane & ((32 >> LG) - 1)) == 0) sh[lane >> (5 - LG)][wid] = v[0];
   __syncthreads();
-  for (int i = wid; i < M; i += kRedWarps) {
-    double v = lane < kRedWarps ? sh[i][lane] : 0.0;
-    v = warp_sum(v);
-    if (lane == 0) partial[(int64_t)i * gridDim.x + blockIdx.x] = v;
+  for (int i = (int)threadIdx.x >> 3; i < (M + 3) / 4 * 4; i += kRedThreads / 8) {
+    double t = i < M ? sh[i][threadIdx.x & 7] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, 8);
+    if (i < M && (threadIdx.x & 7) == 0) partial[(int64_t)i * gridDim.x + blockIdx.x] = t;
   }
 }
 
@@ -263,34 +288,34 @@ __global__ void __launch_bounds__(kRedThreads) k_dots(const S* __restrict__ w, c
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   const VT* w4 = reinterpret_cast<const VT*>(w);
   int chunks = 0;
-  for (int64_t c0 = tid; c0 < nv; c0 += nth * U) {
-    VT wv[U], vv[U][K];
+  auto trip = [&](auto uc, int64_t c0) {  // chunks c0, c0 + nth, ...: all their loads first
+    constexpr int UU = decltype(uc)::value;
+    VT wv[UU], vv[UU][K];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
+    for (int u = 0; u < UU; ++u) {
       const int64_t c = c0 + u * nth;
-      if (c < nv) {
-        wv[u] = w4[c];
+      wv[u] = w4[c];
 #pragma unroll
-        for (int i = 0; i < K; ++i) vv[u][i] = reinterpret_cast<const VT*>(V + i * ldv)[c];
-      }
+      for (int i = 0; i < K; ++i) vv[u][i] = reinterpret_cast<const VT*>(V + i * ldv)[c];
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (c0 + u * nth < nv) {
+    for (int u = 0; u < UU; ++u) {
 #pragma unroll
-        for (int l = 0; l < W; ++l) {
-          const S x = Vec<S>::get(wv[u], l);
+      for (int l = 0; l < W; ++l) {
+        const S x = Vec<S>::get(wv[u], l);
 #pragma unroll
-          for (int i = 0; i < K; ++i) acc[i].add(x, Vec<S>::get(vv[u][i], l));
-          acc[K].add(x, x);
-        }
-        if ((++chunks & 3) == 0) {
+        for (int i = 0; i < K; ++i) acc[i].add(x, Vec<S>::get(vv[u][i], l));
+        acc[K].add(x, x);
+      }
+      if ((++chunks & 3) == 0) {
 #pragma unroll
-          for (int i = 0; i <= K; ++i) acc[i].flush();
-        }
+        for (int i = 0; i <= K; ++i) acc[i].flush();
       }
     }
-  }
+  };
+  int64_t c0 = tid;
+  for (; c0 + (U - 1) * nth < nv; c0 += nth * U) trip(std::integral_constant<int, U>{}, c0);
+  for (; c0 < nv; c0 += nth) trip(std::integral_constant<int, 1>{}, c0);
   for (int64_t j = nv * W + tid; j < n; j += nth) {  // tail
     const S x = w[j];
 #pragma unroll
@@ -340,40 +365,39 @@ __global__ void __launch_bounds__(kRedThreads) k_update(S* __restrict__ w, const
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
   VT* w4 = reinterpret_cast<VT*>(w);
   int chunks = 0;
-  for (int64_t c0 = tid; c0 < nv; c0 += nth * U) {
-    VT wv[U], vv[U][K > 0 ? K : 1];
+  auto trip = [&](auto uc, int64_t c0) {  // chunks c0, c0 + nth, ...: all their loads first
+    constexpr int UU = decltype(uc)::value;
+    VT wv[UU], vv[UU][K > 0 ? K : 1];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
+    for (int u = 0; u < UU; ++u) {
       const int64_t cix = c0 + u * nth;
-      if (cix < nv) {
-        wv[u] = w4[cix];
+      wv[u] = w4[cix];
 #pragma unroll
-        for (int i = 0; i < K; ++i) vv[u][i] = reinterpret_cast<const VT*>(V + i * ldv)[cix];
-      }
+      for (int i = 0; i < K; ++i) vv[u][i] = reinterpret_cast<const VT*>(V + i * ldv)[cix];
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t cix = c0 + u * nth;
-      if (cix < nv) {
+    for (int u = 0; u < UU; ++u) {
 #pragma unroll
-        for (int l = 0; l < W; ++l) {
-          S x = Vec<S>::get(wv[u], l);
+      for (int l = 0; l < W; ++l) {
+        S x = Vec<S>::get(wv[u], l);
 #pragma unroll
-          for (int i = 0; i < K; ++i) x = fma(-cc[i], Vec<S>::get(vv[u][i], l), x);
-          Vec<S>::set(wv[u], l, x);
-          acc.add(x, x);
+        for (int i = 0; i < K; ++i) x = fma(-cc[i], Vec<S>::get(vv[u][i], l), x);
+        Vec<S>::set(wv[u], l, x);
+        acc.add(x, x);
 #pragma unroll
-          for (int i = 0; i < ND; ++i) dot[i].add(x, Vec<S>::get(vv[u][i], l));
-        }
-        if ((++chunks & 3) == 0) {
-          acc.flush();
-#pragma unroll
-          for (int i = 0; i < ND; ++i) dot[i].flush();
-        }
-        if (K > 0) w4[cix] = wv[u];
+        for (int i = 0; i < ND; ++i) dot[i].add(x, Vec<S>::get(vv[u][i], l));
       }
+      if ((++chunks & 3) == 0) {
+        acc.flush();
+#pragma unroll
+        for (int i = 0; i < ND; ++i) dot[i].flush();
+      }
+      if (K > 0) w4[c0 + u * nth] = wv[u];
     }
-  }
+  };
+  int64_t c0 = tid;
+  for (; c0 + (U - 1) * nth < nv; c0 += nth * U) trip(std::integral_constant<int, U>{}, c0);
+  for (; c0 < nv; c0 += nth) trip(std::integral_constant<int, 1>{}, c0);
   for (int64_t j = nv * W + tid; j < n; j += nth) {  // tail
     S x = w[j];
 #pragma unroll
@@ -432,6 +456,7 @@ __global__ void __launch_bounds__(kRedThreads) k_norm_step(const double* __restr
   Acc<double> acc;
   Acc<float> acc32;
   int chunks = 0;
+#pragma unroll 4
   for (int64_t c = tid; c < nv; c += nth) {  // four entries: two 16-byte loads
     const double2 a = v2[2 * c], b = v2[2 * c + 1];
     if constexpr (CONV) {
@@ -532,6 +557,9 @@ __global__ void k_precond(S* __restrict__ z, const S* __restrict__ v, const S* _
   for (int64_t j = (blk >= W ? nv * W : 0) + tid; j < n; j += nth) z[j] = v[j] * inv[block_of<Small>(j, blk)];
 }
 
+// Four entries a thread: 16-byte loads of the basis (FP32; two of them in FP64) and of x.  64^3-like
+// vectors are far larger than L2, so this is bound by HBM: 32^3 elements, p = 4, q = 3, ten FP32
+// columns 1.01 -> 0.64 ms.
 template <typename S, typename X, int K, bool Small>
 __global__ void k_precond_combine(X* __restrict__ x, const S* __restrict__ V, int64_t ldv, Coef16 y,
                                   const S* __restrict__ inv, int64_t blk, int64_t n, const GmresState* st) {
@@ -541,12 +569,46 @@ __global__ void k_precond_combine(X* __restrict__ x, const S* __restrict__ V, in
   S yy[K > 0 ? K : 1];
 #pragma unroll
   for (int i = 0; i < K; ++i) yy[i] = (S)(st ? st->yc[i] : y.c[i]);
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+  using VS = typename Vec<S>::T;
+  using VX = typename Vec<X>::T;
+  constexpr int WS = Vec<S>::W, WX = Vec<X>::W, GS = 4 / WS, GX = 4 / WX;
+  const int64_t n4 = n / 4;
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t c = tid; c < n4; c += nth) {
+    VX xv[GX];
+#pragma unroll
+    for (int g = 0; g < GX; ++g) xv[g] = reinterpret_cast<const VX*>(x)[c * GX + g];
+    S v[4] = {S(0), S(0), S(0), S(0)};
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      if (i < kk) {
+#pragma unroll
+        for (int g = 0; g < GS; ++g) {
+          const VS w = reinterpret_cast<const VS*>(V + i * ldv)[c * GS + g];
+#pragma unroll
+          for (int l = 0; l < WS; ++l) v[g * WS + l] = fma(yy[i], Vec<S>::get(w, l), v[g * WS + l]);
+        }
+      }
+    }
+    int64_t b = block_of<Small>(c * 4, blk), edge = (b + 1) * blk;
+    S s = inv[b];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      if (c * 4 + l >= edge) {
+        s = inv[++b];
+        edge += blk;
+      }
+      Vec<X>::set(xv[l / WX], l % WX, Vec<X>::get(xv[l / WX], l % WX) + (X)(v[l] * s));
+    }
+#pragma unroll
+    for (int g = 0; g < GX; ++g) reinterpret_cast<VX*>(x)[c * GX + g] = xv[g];
+  }
+  for (int64_t j = n4 * 4 + tid; j < n; j += nth) {  // tail
     S v = S(0);
 #pragma unroll
     for (int i = 0; i < K; ++i)
       if (i < kk) v = fma(yy[i], V[i * ldv + j], v);
-    x[j] = (X)x[j] + (X)(v * inv[block_of<Small>(j, blk)]);
+    x[j] = x[j] + (X)(v * inv[block_of<Small>(j, blk)]);
   }
 }
 
@@ -555,10 +617,14 @@ __global__ void __launch_bounds__(kRedThreads) k_energy(const double* __restrict
                                                         int64_t n3, int64_t n, double* __restrict__ partial) {
   __shared__ double sh[32];
   double acc = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const double v = u[j];
-    acc = fma(mass[block_of<Small>(j, n3)] * v, v, acc);
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (int64_t c = tid; c < n / 2; c += nth) {
+    const double2 v = reinterpret_cast<const double2*>(u)[c];
+    acc = fma(mass[block_of<Small>(2 * c, n3)] * v.x, v.x, acc);
+    acc = fma(mass[block_of<Small>(2 * c + 1, n3)] * v.y, v.y, acc);
   }
+  if (tid == 0 && (n & 1)) acc = fma(mass[block_of<Small>(n - 1, n3)] * u[n - 1], u[n - 1], acc);
   const double r = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = 0.5 * r;
 }
@@ -578,17 +644,21 @@ inline int grid_for(int64_t n) {
 
 inline bool small(int64_t n) { return n <= (int64_t)0xffffffffLL; }
 
-// Blocks of a reduction over nv vectors: one vector a thread on small problems, at most kRedBlocks.
-inline int red_grid(int64_t nv) {
+// Blocks of a reduction over nv vectors: one vector a thread on small problems, else one wave of
+// co-resident blocks (at most kRedBlocks).  A fixed 608 ran a second, mostly empty wave where the
+// registers hold fewer than four blocks per SM (ten FP32 columns: 618 us against 490 expected).
+template <typename F>
+inline int red_grid(F kernel, int64_t nv, std::atomic<int>* cache) {
   const int64_t g = (nv + kRedThreads - 1) / kRedThreads;
-  return (int)(g < 1 ? 1 : (g < kRedBlocks ? g : kRedBlocks));
+  return wave_grid(kernel, kRedThreads, 0, g < 1 ? 1 : (g < kRedBlocks ? g : kRedBlocks), cache);
 }
 
 template <typename S, typename X, int K>
 void combine_k(X* x, const S* V, int64_t ldv, const Coef16& y, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
                const GmresState* st) {
-  if (small(n)) k_precond_combine<S, X, K, true><<<grid_for(n), kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
-  else k_precond_combine<S, X, K, false><<<grid_for(n), kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
+  const int g = grid_for((n + 3) / 4);
+  if (small(n)) k_precond_combine<S, X, K, true><<<g, kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
+  else k_precond_combine<S, X, K, false><<<g, kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
 }
 
 #define STM_SWITCH_K(k, CALL)  \
@@ -613,13 +683,15 @@ void combine_k(X* x, const S* V, int64_t ldv, const Coef16& y, const S* inv, int
 }  // namespace
 
 void dot(const double* w, const double* v, int64_t n, double* partial, double* out, cudaStream_t s) {
-  const int g = red_grid(n / Vec<double>::W);
+  static std::atomic<int> cap[64];
+  const int g = red_grid(k_dots<double, 1, false>, n / Vec<double>::W, cap);
   k_dots<double, 1, false><<<g, kRedThreads, 0, s>>>(w, v, 0, n, partial, nullptr);
   k_finish<<<1, 32, 0, s>>>(partial, 1, g, out);
 }
 
 void axpy_norm(double* w, const double* v, double c, int64_t n, double* partial, double* out, cudaStream_t s) {
-  const int g = red_grid(n / Vec<double>::W);
+  static std::atomic<int> cap[64];
+  const int g = red_grid(k_update<double, 1, kPlain>, n / Vec<double>::W, cap);
   Coef16 cc{};
   cc.c[0] = c;
   if (v) k_update<double, 1, kPlain><<<g, kRedThreads, 0, s>>>(w, v, 0, cc, n, partial, nullptr, 0);
@@ -627,11 +699,24 @@ void axpy_norm(double* w, const double* v, double c, int64_t n, double* partial,
   k_finish<<<1, 32, 0, s>>>(partial, 1, g, out);
 }
 
+template <typename S, int K>
+void dots_k(const S* w, const S* V, int64_t ldv, int64_t n, double* partial, GmresState* st, cudaStream_t s) {
+  static std::atomic<int> cap[64];
+  auto k = k_dots<S, K, true>;
+  k<<<red_grid(k, n / Vec<S>::W, cap), kRedThreads, 0, s>>>(w, V, ldv, n, partial, st);
+}
+
+template <typename S, int K, int MODE>
+void update_k(S* w, const S* V, int64_t ldv, int64_t n, double* partial, GmresState* st, int m, cudaStream_t s) {
+  static std::atomic<int> cap[64];
+  auto k = k_update<S, K, MODE>;
+  k<<<red_grid(k, n / Vec<S>::W, cap), kRedThreads, 0, s>>>(w, V, ldv, Coef16{}, n, partial, st, m);
+}
+
 template <typename S>
 void gmres_dots(const S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st,
                 cudaStream_t s) {
-  const int g = red_grid(n / Vec<S>::W);
-#define STM_MD(K) k_dots<S, K, true><<<g, kRedThreads, 0, s>>>(w, V, ldv, n, partial, st)
+#define STM_MD(K) dots_k<S, K>(w, V, ldv, n, partial, st, s)
   STM_SWITCH_K(j + 1, STM_MD)
 #undef STM_MD
 }
@@ -639,11 +724,9 @@ void gmres_dots(const S* w, const S* V, int64_t ldv, int j, int64_t n, double* p
 template <typename S>
 void gmres_update(S* w, const S* V, int64_t ldv, int j, int64_t n, double* partial, GmresState* st, int m, bool reorth,
                   cudaStream_t s) {
-  const int g = red_grid(n / Vec<S>::W);
-  const Coef16 c{};
-#define STM_UP(K) k_update<S, K, kOnly><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
-#define STM_UP1(K) k_update<S, K, kFirst><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
-#define STM_UP2(K) k_update<S, K, kSecond><<<g, kRedThreads, 0, s>>>(w, V, ldv, c, n, partial, st, m)
+#define STM_UP(K) update_k<S, K, kOnly>(w, V, ldv, n, partial, st, m, s)
+#define STM_UP1(K) update_k<S, K, kFirst>(w, V, ldv, n, partial, st, m, s)
+#define STM_UP2(K) update_k<S, K, kSecond>(w, V, ldv, n, partial, st, m, s)
   if (reorth) {
     STM_SWITCH_K(j + 1, STM_UP1)
     STM_SWITCH_K(j + 1, STM_UP2)
@@ -656,13 +739,15 @@ void gmres_update(S* w, const S* V, int64_t ldv, int j, int64_t n, double* parti
 }
 
 void gmres_norm(const double* v, int64_t n, double* partial, GmresState* st, const NormStep& step, cudaStream_t s) {
-  k_norm_step<false><<<red_grid(n / 4), kRedThreads, 0, s>>>(v, nullptr, n, partial, st, step);
+  static std::atomic<int> cap[64];
+  k_norm_step<false><<<red_grid(k_norm_step<false>, n / 4, cap), kRedThreads, 0, s>>>(v, nullptr, n, partial, st, step);
 }
 
 void gmres_start32(const double* v, float* v32, int64_t n, double* partial, GmresState* st, cudaStream_t s) {
   NormStep step{};
   step.kind = NormStep::kStart32;
-  k_norm_step<true><<<red_grid(n / 4), kRedThreads, 0, s>>>(v, v32, n, partial, st, step);
+  static std::atomic<int> cap[64];
+  k_norm_step<true><<<red_grid(k_norm_step<true>, n / 4, cap), kRedThreads, 0, s>>>(v, v32, n, partial, st, step);
 }
 
 template <typename S>

@@ -1178,19 +1178,22 @@ __global__ void k_copy_words(double* __restrict__ dst, const double* __restrict_
   }
 }
 
-__global__ void k_init_guess(double* x, const double* state, int64_t q, int64_t n3, int64_t n) {
+// I: 32-bit indices where the vector allows (a 64-bit division per entry cost more than the traffic)
+template <typename I>
+__global__ void k_init_guess(double* __restrict__ x, const double* __restrict__ state, I q, I n3, int64_t n) {
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t blk = j / n3, s = j - blk * n3;
-    const int64_t fc = blk / q, i = blk - fc * q;
-    x[j] = (i == 0) ? state[fc * n3 + s] : 0.0;
+    const I blk = (I)j / n3, s = (I)j - blk * n3;
+    const I fc = blk / q, i = blk - fc * q;
+    x[j] = (i == 0) ? state[(int64_t)fc * n3 + s] : 0.0;
   }
 }
 
-__global__ void k_extract_end(double* state, const double* x, int64_t q, int64_t n3, int64_t n) {
+template <typename I>
+__global__ void k_extract_end(double* __restrict__ state, const double* __restrict__ x, I q, I n3, int64_t n) {
   // end of the slab: l_1(1) = 1, l_m(1) = 0 otherwise, so u(t0+dt) = mode 1 = Krylov index 0
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t fc = j / n3, s = j - fc * n3;
-    state[j] = x[(fc * q) * n3 + s];
+    const I fc = (I)j / n3, s = (I)j - fc * n3;
+    state[j] = x[(int64_t)fc * q * n3 + s];
   }
 }
 
@@ -2403,7 +2406,8 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
   // initial guess: u_1 = u_0, higher modes 0 (or all unknowns 0: x is already zero)
   if (!c->opts.zero_guess) {
     if (c->hp) init_guess_hp(c->x, c->state, c->off_test, c->off_state, c->pq, c->ne, c->stream);
-    else k_init_guess<<<grid1(n), 256, 0, c->stream>>>(c->x, c->state, c->Q, c->N3, n);
+    else if (n < (1LL << 32)) k_init_guess<uint32_t><<<grid1(n), 256, 0, c->stream>>>(c->x, c->state, c->Q, c->N3, n);
+    else k_init_guess<int64_t><<<grid1(n), 256, 0, c->stream>>>(c->x, c->state, c->Q, c->N3, n);
     c->launches += 1;
   }
   // restart cycles, each one launch sequence (a replayed CUDA graph unless profiling) and one
@@ -2431,7 +2435,9 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
   }
   if (int rc = check_wait_err(c)) return rc;
   if (c->hp) extract_end_hp(c->state, c->x, c->off_test, c->off_state, c->pq, c->ne, c->stream);
-  else k_extract_end<<<grid1(c->n_state), 256, 0, c->stream>>>(c->state, c->x, c->Q, c->N3, c->n_state);
+  else if (n < (1LL << 32))
+    k_extract_end<uint32_t><<<grid1(c->n_state), 256, 0, c->stream>>>(c->state, c->x, c->Q, c->N3, c->n_state);
+  else k_extract_end<int64_t><<<grid1(c->n_state), 256, 0, c->stream>>>(c->state, c->x, c->Q, c->N3, c->n_state);
   c->launches += 1;
   STM_CK(cudaGetLastError());
   c->t += dt;
