@@ -1,5 +1,7 @@
 #include "hp.cuh"
 
+#include "residual.cuh"
+
 namespace stm {
 
 namespace {
@@ -96,41 +98,54 @@ __global__ void k_energy_hp(const double* __restrict__ u, const double* __restri
   }
 }
 
+// One slot per block.  The two tangential transfers are applied one after the other through shared
+// memory, row by row (Ns) then column by column, so a value takes 2 Ns products instead of Ns^2; the
+// transfer integrals sit in shared memory (lanes read different entries, which a constant bank
+// serialises).  The launch runs alone between the trace and the apply passes; octree of 45,123 elements,
+// p <= 7, q <= 4: FP64 apply 3.00 -> 2.84 ms, FP32 operator 1.35 -> 1.25 ms
+constexpr int kHangPlanes = 4 * kMaxQ;
 template <typename T>
 __global__ void __launch_bounds__(128) k_hang(HangArgs<T> H) {
   if (H.skip && *H.skip) return;
+  __shared__ T Tm[2][8][8], tmp[kHangPlanes][8][8], out[kHangPlanes][8][8];
+  for (int k = threadIdx.x; k < 128; k += blockDim.x) (&Tm[0][0][0])[k] = (&H.Tm[0][0][0])[k];
   for (int64_t slot = blockIdx.x; slot < H.n_slots; slot += gridDim.x) {
-    const int e = H.elem[slot], face = H.face[slot], a = face >> 1;
-    int n3, q;
-    degrees(H.pq, e, n3, q);
-    const int N = (H.pq[e] & 15) + 1, N2 = N * N;
-    const int kind = H.kind[slot];
-    for (int it = threadIdx.x; it < 4 * q * N2; it += blockDim.x) {
-      const int t = it % N2, r = it / N2, i = r % q, fb = r / q;  // fb = field * 2 + comp slot
-      const int fld = fb >> 1, bi = fb & 1;
-      const int js = t / N, jf = t - js * N;
-      T acc = T(0);
-      const int nsrc = kind == 0 ? 1 : 4;
-      for (int k = 0; k < nsrc; ++k) {
-        const int es = H.src[slot * 4 + k], sf = H.src_face[slot * 4 + k];
-        const int qs = H.pq[es] >> 4, Ns = (H.pq[es] & 15) + 1;
-        if (i >= qs) continue;
-        const int u = H.quad[slot * 4 + k] & 1, v = H.quad[slot * 4 + k] >> 1;
-        const T* ts = H.tr + H.off_tr[es] + ((((int64_t)fld * 3 + a) * 2 + (sf & 1)) * 2 + bi) * qs * Ns * Ns +
-                      (int64_t)i * Ns * Ns;
-        for (int ns = 0; ns < Ns; ++ns) {
-          T row = T(0);
-          for (int nf = 0; nf < Ns; ++nf) {
-            // fine side: source modes (ns, nf) are the coarse ones; coarse side: they are fine ones
-            const T tf = kind == 0 ? H.Tm[u][jf][nf] : H.Tm[u][nf][jf];
-            row = fma(tf, ts[ns * Ns + nf], row);
-          }
-          const T tsl = kind == 0 ? H.Tm[v][js][ns] : H.Tm[v][ns][js];
-          acc = fma(tsl, row, acc);
-        }
+    const int e = H.elem[slot], a = H.face[slot] >> 1;
+    const int N = (H.pq[e] & 15) + 1, q = H.pq[e] >> 4, N2 = N * N;
+    const int kind = H.kind[slot], nsrc = kind == 0 ? 1 : 4;
+    for (int it = threadIdx.x; it < 4 * q * 64; it += blockDim.x) (&out[0][0][0])[it] = T(0);
+    __syncthreads();
+    for (int k = 0; k < nsrc; ++k) {
+      const int es = H.src[slot * 4 + k], sf = H.src_face[slot * 4 + k];
+      const int qs = H.pq[es] >> 4, Ns = (H.pq[es] & 15) + 1, qm = qs < q ? qs : q;
+      const int u = H.quad[slot * 4 + k] & 1, v = H.quad[slot * 4 + k] >> 1;
+      const T* ts = H.tr + H.off_tr[es];
+      // planes fb * qm + i, fb = field * 2 + comp slot: the fast axis
+      for (int it = threadIdx.x; it < 4 * qm * Ns * N; it += blockDim.x) {
+        const int jf = it % N, r = it / N, ns = r % Ns, pl = r / Ns, fb = pl / qm, i = pl - fb * qm;
+        const int so = ((((fb >> 1) * 3 + a) * 2 + (sf & 1)) * 2 + (fb & 1)) * qs + i;
+        const T* row = ts + (int64_t)so * (Ns * Ns) + ns * Ns;
+        T acc = T(0);
+        // fine side: the source modes are the coarse ones; coarse side: they are fine ones
+        for (int nf = 0; nf < Ns; ++nf) acc = fma(kind == 0 ? Tm[u][jf][nf] : Tm[u][nf][jf], row[nf], acc);
+        tmp[pl][ns][jf] = acc;
       }
-      H.hbuf[H.hoff[slot] + it] = T(0.5) * acc;
+      __syncthreads();
+      // the slow axis, added to the receiving element's planes fb * q + i
+      for (int it = threadIdx.x; it < 4 * qm * N2; it += blockDim.x) {
+        const int jf = it % N, r = it / N, js = r % N, pl = r / N, fb = pl / qm, i = pl - fb * qm;
+        T acc = out[fb * q + i][js][jf];
+        for (int ns = 0; ns < Ns; ++ns) acc = fma(kind == 0 ? Tm[v][js][ns] : Tm[v][ns][js], tmp[pl][ns][jf], acc);
+        out[fb * q + i][js][jf] = acc;
+      }
+      __syncthreads();
     }
+    T* o = H.hbuf + H.hoff[slot];
+    for (int it = threadIdx.x; it < 4 * q * N2; it += blockDim.x) {
+      const int t = it % N2, pl = it / N2, js = t / N;
+      o[it] = T(0.5) * out[pl][js][t - js * N];
+    }
+    __syncthreads();
   }
 }
 
