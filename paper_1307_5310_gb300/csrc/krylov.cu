@@ -156,6 +156,7 @@ __device__ void grid_sums(const double* __restrict__ partial, int m, double* out
 // ---- scalar steps of the device-side GMRES control, run by the last block of a reduction ----
 
 __device__ void outer_check(GmresState* st) {
+  st->used = st->k;
   st->k = 0;
   st->skip_reo = 1;
   const double beta = sqrt(st->red[0]);
@@ -444,6 +445,7 @@ __global__ void __launch_bounds__(kRedThreads) k_norm_step(const double* __restr
   } else if (st->halt) {
     // the slab has stopped: this cycle applies nothing
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+      st->used = st->k;
       st->k = 0;
       st->skip = 1;
       st->skip_reo = 1;

@@ -42,6 +42,7 @@ struct GmresState {
   double tol_abs;                 // this cycle's stop threshold on |g|
   double rel, phi, res;           // last true relative residual, weighted norm, |g_k|
   int32_t k;                      // basis vectors used in this cycle
+  int32_t used;                   // those of the cycle before the last stop test
   int32_t skip;                   // 1: the rest of the cycle is skipped
   int32_t skip_reo;               // 1: no second Gram-Schmidt pass in this iteration
   int32_t iters;                  // GMRES iterations of the slab so far
