@@ -1293,6 +1293,15 @@ __host__ __device__ constexpr size_t fused_smem(int P, int Q) {
   return sizeof(float) * (2 * 6 * Q * (P + 1) * (P + 1) * (P + 1) + 24 * Q * (P + 1) * (P + 1));
 }
 __host__ __device__ constexpr bool fused_fits(int P, int Q) { return fused_smem(P, Q) <= 64 * 1024; }
+// Whether a uniform FP32 mesh runs it.  A CTA of six warps per element is mostly idle on the smallest
+// elements, where blocks of 64 threads in two kernels are faster once the mesh fills the GPU; on small
+// meshes the single launch is.  FP32 operator, single pass against two kernels: p = 1, q = 1 12^3
+// elements 33 / 36 us, 20^3 58 / 42, 80^3 2,100 / 909; p = 1, q = 6 40^3 517 / 258; p = 2, q = 3 12^3
+// 36 / 39; p = 2, q = 4 40^3 497 / 421; p = 2, q = 6 24^3 159 / 148 (residual 121 / 129); p = 3, q = 2
+// 48^3 757 / 712 (residual 676 / 722); p = 3, q = 4 40^3 644 / 758.
+constexpr bool single_pass32(int P, int Q, int64_t n_elem) {
+  return fused_fits(P, Q) && !(P <= 1 && n_elem >= 4096) && !(P == 2 && Q <= 4 && n_elem >= 32768);
+}
 
 template <typename T, int P, int Q>
 int launch_residual_pq(const ApplyArgs<T>& args, cudaStream_t s, int grid, const LaunchEvents& ev, int phase = 0,
@@ -1331,7 +1340,7 @@ int launch_residual_pq(const ApplyArgs<T>& args, cudaStream_t s, int grid, const
   });
   const bool hp = args.elist != nullptr;
   if constexpr (sizeof(T) == 4 && fused_fits(P, Q)) {
-    if (!hp) {
+    if (!hp && single_pass32(P, Q, args.n_elem)) {
       // single pass: ev.start/ev.stop bracket k_fused (reported in the apply slot)
       if (ev.start) cudaEventRecord(ev.start, s);
       if (ev.mid) cudaEventRecord(ev.mid, s);

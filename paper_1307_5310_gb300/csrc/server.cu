@@ -24,6 +24,7 @@
 #include <thread>
 #include <vector>
 
+#include "residual.cuh"
 #include "stm.h"
 
 namespace {
@@ -78,8 +79,12 @@ int64_t footprint(const stm_request& r, const stm_server_opts& o) {
   const int64_t test = ne * 6 * r.q * n3, state = ne * 6 * n3, tr = ne * 24 * r.q * n2;
   const int64_t m = o.restart;
   int64_t b = 8 * (test + tr) + 8 * 2 * state + 8 * 2 * test + 8 * test + 4 * test + ne * 512;
-  if (o.precision == STM_MIXED) b += 4 * (m + 1) * test + 4 * test;
-  else b += 8 * (m + 1) * test;
+  if (o.precision == STM_MIXED) {
+    b += 4 * (m + 1) * test + 4 * test;
+    if (!stm::single_pass32(r.p, r.q, ne)) b += 4 * (test + tr);  // FP32 scratch of the two-kernel passes
+  } else {
+    b += 8 * (m + 1) * test;
+  }
   return b + (64 << 20);
 }
 

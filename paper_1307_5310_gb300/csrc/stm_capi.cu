@@ -434,10 +434,10 @@ const T* kap_ptr(stm_ctx* c) {
 }
 
 // Whether the residual kernels of precision T use the y / trace scratch: all but the
-// single-pass FP32 kernel (uniform meshes, with or without D_h, shared memory within fused_fits).
+// single-pass FP32 kernel (uniform meshes, with or without D_h, by the rule of single_pass32).
 template <typename T>
 bool needs_scratch(const stm_ctx* c) {
-  return sizeof(T) == 8 || c->hp || !fused_fits(c->P, c->Q);
+  return sizeof(T) == 8 || c->hp || !single_pass32(c->P, c->Q, c->ne);
 }
 
 // Upper bound of the residual kernels' grids (grid-stride loops over elements): the launch

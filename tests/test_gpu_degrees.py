@@ -60,6 +60,15 @@ def test_every_degree(mods, geom, p):
         _check(mods, m, 0.04)
 
 
+@pytest.mark.parametrize("n,p,q", [((16, 16, 15), 1, 1), ((16, 16, 16), 1, 1), ((16, 16, 16), 0, 3),
+                                   ((32, 32, 31), 2, 1), ((32, 32, 32), 2, 1), ((32, 33, 32), 2, 4)])
+def test_low_degree_mesh_sizes(mods, n, p, q):
+    """Either side of the sizes where low-degree FP32 meshes change from one kernel to two."""
+    m = meshgen.box_mesh(*n, hi=(1.0, 0.8, 1.2), p=p, q=q)
+    meshgen.random_materials(m, 81, 82)
+    _check(mods, m, 0.01)
+
+
 @pytest.mark.parametrize("qmax", [2, 6])
 def test_uneven_degrees_and_partitions(mods, qmax):
     m = meshgen.corner_octree_mesh(3, [0.7, 0.3])
