@@ -1340,7 +1340,7 @@ int launch_residual_pq(const ApplyArgs<T>& args, cudaStream_t s, int grid, const
   });
   const bool hp = args.elist != nullptr;
   if constexpr (sizeof(T) == 4 && fused_fits(P, Q)) {
-    if (!hp && single_pass32(P, Q, args.n_elem)) {
+    if (!hp && (single_pass32(P, Q, args.n_elem) || !args.y)) {  // y null: no scratch to be had
       // single pass: ev.start/ev.stop bracket k_fused (reported in the apply slot)
       if (ev.start) cudaEventRecord(ev.start, s);
       if (ev.mid) cudaEventRecord(ev.mid, s);

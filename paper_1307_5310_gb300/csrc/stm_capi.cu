@@ -342,10 +342,14 @@ int ensure_scratch(stm_ctx* c, T** y, T** tr) {
   if (*y) return STM_OK;
   const size_t ny = (size_t)c->n_test;
   const size_t nt = (size_t)c->n_tr;
-  if (cudaMalloc((void**)y, ny * sizeof(T)) != cudaSuccess || cudaMalloc((void**)tr, nt * sizeof(T)) != cudaSuccess) {
+  T *py = nullptr, *pt = nullptr;
+  if (cudaMalloc((void**)&py, ny * sizeof(T)) != cudaSuccess || cudaMalloc((void**)&pt, nt * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
+    if (py) cudaFree(py);  // both or neither: the next call tries again
     return fail(c, STM_ENOMEM, "scratch allocation failed");
   }
+  *y = py;
+  *tr = pt;
   return STM_OK;
 }
 
@@ -440,6 +444,28 @@ bool needs_scratch(const stm_ctx* c) {
   return sizeof(T) == 8 || c->hp || !single_pass32(c->P, c->Q, c->ne);
 }
 
+// The scratch of a residual launch (null where it needs none).  Uniform FP32 meshes that are faster in
+// two kernels but also fit the single pass run that one while the scratch cannot be had: on a stream
+// being captured before it exists, or when the allocation fails.
+template <typename T>
+int residual_scratch(stm_ctx* c, T** y, T** tr) {
+  *y = *tr = nullptr;
+  if (!needs_scratch<T>(c)) return STM_OK;
+  const bool optional = sizeof(T) == 4 && !c->hp && fused_fits(c->P, c->Q);
+  if (optional && !c->y32) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    STM_CK(cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return STM_OK;
+  }
+  const int rc = scratch<T>(c, y, tr);
+  if (rc && optional) {
+    *y = *tr = nullptr;
+    c->err.clear();
+    return STM_OK;
+  }
+  return rc;
+}
+
 // Upper bound of the residual kernels' grids (grid-stride loops over elements): the launch
 // sizes each grid to one wave of co-resident CTAs (wave_grid in residual.cuh).
 int res_grid(const stm_ctx* c, int64_t count) {
@@ -493,8 +519,8 @@ template <typename T>
 int apply(stm_ctx* c, double dt, const T* um, int um_layout, const T* u0, int u0_layout, const T* b, T* R,
           bool pre = false, const int32_t* skip = nullptr) {
   T *y = nullptr, *tr = nullptr;
-  if (needs_scratch<T>(c)) {  // the uniform FP32 single-pass kernel needs none
-    int rc = scratch<T>(c, &y, &tr);
+  {
+    const int rc = residual_scratch<T>(c, &y, &tr);
     if (rc) return rc;
   }
   ApplyArgs<T> a{};
@@ -2387,9 +2413,9 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
     }
     STM_CK(cudaMemsetAsync(c->gst, 0, sizeof(GmresState), c->stream));
   }
-  if (mixed && needs_scratch<float>(c)) {  // FP32 residual scratch, allocated before any capture
+  if (mixed) {  // FP32 residual scratch, allocated before any capture
     float *y32 = nullptr, *tr32 = nullptr;
-    if ((rc = scratch<float>(c, &y32, &tr32))) return rc;
+    if ((rc = residual_scratch<float>(c, &y32, &tr32))) return rc;
   }
   const double* b = nullptr;
   if ((rc = build_load(c, c->t, dt, &b))) return rc;

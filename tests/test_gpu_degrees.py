@@ -69,6 +69,38 @@ def test_low_degree_mesh_sizes(mods, n, p, q):
     _check(mods, m, 0.01)
 
 
+def test_first_apply_under_capture(mods):
+    """A low-degree FP32 mesh whose first apply is captured (no scratch may be allocated then) runs the
+    single pass; later applies run the two kernels.  Both against the FP64 evaluation, bar 2e-6."""
+    import torch
+
+    stm, cases = mods
+    m = meshgen.box_mesh(16, p=1, q=1)
+    meshgen.random_materials(m, 83, 84)
+    dt = 0.01
+    x = cases._Exact(m, dt)
+    side = torch.cuda.Stream()
+    s = stm.Slab(m, stream=side.cuda_stream)
+    U = torch.empty(s.n_trial, dtype=torch.float64, device="cuda").uniform_(-1, 1)
+    u, out = U.float(), torch.zeros(s.n_test, dtype=torch.float32, device="cuda")
+    ref = x.residual(x.gather(U, True))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        s.residual_apply(u, out, 0.0, dt, prec=stm.STM_FP32)
+    g.replay()
+    torch.cuda.synchronize()
+    assert float((out.double() - ref).norm() / ref.norm()) < 2e-6
+    out.zero_()
+    torch.cuda.synchronize()
+    s.residual_apply(u, out, 0.0, dt, prec=stm.STM_FP32)
+    torch.cuda.synchronize()
+    assert float((out.double() - ref).norm() / ref.norm()) < 2e-6
+    g.replay()
+    torch.cuda.synchronize()
+    assert float((out.double() - ref).norm() / ref.norm()) < 2e-6
+
+
 @pytest.mark.parametrize("qmax", [2, 6])
 def test_uneven_degrees_and_partitions(mods, qmax):
     m = meshgen.corner_octree_mesh(3, [0.7, 0.3])
