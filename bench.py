@@ -89,12 +89,13 @@ def workload(n, p, q):
 def flops_per_element(p, q):
     """Algorithmic flops of one residual apply per element (both fields), split by kernel.
 
-    prep : y = B u (nnzB per point) and the folded face traces (one pass per axis, 2 comps)
+    prep : unnormalised moments (1 per point at q = 1, else q + 1) and the folded face traces (one
+           pass per axis, 2 comps, n per line)
     apply: mass (1 FMA per entry), volume curl (6 terms x nnzD per line), folded lift.
     """
     n = p + 1
     n2, n3 = n * n, n ** 3
-    nnzB = 2 if q == 1 else 2 * q + 1
+    nnzB = 1 if q == 1 else q + 1
     nnzD = n * n // 4
     prep = 2 * (3 * n3 * nnzB + 3 * 2 * q * n3)
     apply = 2 * (3 * q * n3 + 6 * q * n2 * nnzD + 3 * 2 * q * n3)
@@ -290,7 +291,10 @@ def curved_flops_per_element(p, q):
     n, nq = p + 1, p + 2
     fl_prep, fl_apply = flops_per_element(p, q)
     affine_mass = 2 * 2 * (3 * q * n ** 3)
-    mass = 2 * 2 * q * (6 * (n ** 3 * nq + n ** 2 * nq ** 2 + n * nq ** 3) + 9 * nq ** 3)
+    # 1-D contractions with the even/odd symmetry of the Gauss points, per line forward and back
+    h, c, ne = nq // 2, nq % 2, (n + 1) // 2
+    line = h * n + c * (ne - 1) + 2 * h + (h - 1 + c) + (ne - 1) * (h + c) + (n // 2) * h
+    mass = 2 * 2 * q * (3 * (n * n + n * nq + nq * nq) * line + 9 * nq ** 3 + 3 * n ** 3)
     return fl_prep, fl_apply - affine_mass, mass
 
 
