@@ -108,7 +108,8 @@ typedef struct {
   double tol;            /* relative residual target of the slab solve            */
   int32_t restart;       /* GMRES restart length n_r (Sec. 5.4: 10)               */
   int32_t max_it;        /* iteration cap per slab                                */
-  int32_t deterministic; /* 1: fixed-order reductions (bitwise reproducible)      */
+  int32_t deterministic; /* 1: fixed-order reductions (bitwise reproducible; see
+                            stm_residual_apply for FP32 applies of low degree)    */
   int64_t stream;        /* cudaStream_t as integer; 0 = the CUDA default stream  */
   int32_t reorth;        /* 1: second Gram-Schmidt pass when the norm drops below
                             1/sqrt(2) of its value (DGKS test); 0: never           */
@@ -167,7 +168,13 @@ int32_t stm_sizes(stm_ctx *ctx, int64_t *n_trial, int64_t *n_test, int64_t *n_st
  * basis function V, with B_h = C_h + S_h (Eq. bilinearform:C, bilinearform:S)
  * on the slab (t0, t0 + dt].  U: trial layout, R: test layout, both of type
  * double (prec = STM_FP64) or float (prec = STM_FP32).  Boundary data and
- * sources set with stm_set_* enter through L; by default g = 0 (PEC), J = 0. */
+ * sources set with stm_set_* enter through L; by default g = 0 (PEC), J = 0.
+ * FP32 applies (this call and stm_operator_apply) of uniform meshes with
+ * p <= 1 and 4,096 or more elements, or p = 2, q <= 4 and 32,768 or more, run
+ * two kernels through scratch the context allocates on the first of them; on a
+ * stream that is being captured, and for the rest of the context's life once
+ * that memory could not be had or was needed for another call, they run one
+ * kernel without scratch, whose results differ by rounding. */
 int32_t stm_residual_apply(stm_ctx *ctx, double t0, double dt, const void *U, void *R,
                            int32_t prec, int32_t mem);
 

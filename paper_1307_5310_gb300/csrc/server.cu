@@ -81,7 +81,7 @@ int64_t footprint(const stm_request& r, const stm_server_opts& o) {
   int64_t b = 8 * (test + tr) + 8 * 2 * state + 8 * 2 * test + 8 * test + 4 * test + ne * 512;
   if (o.precision == STM_MIXED) {
     b += 4 * (m + 1) * test + 4 * test;
-    if (!stm::single_pass32(r.p, r.q, ne)) b += 4 * (test + tr);  // FP32 scratch of the two-kernel passes
+    if (!stm::fused_fits(r.p, r.q)) b += 4 * (test + tr);  // FP32 scratch of the two-kernel passes
   } else {
     b += 8 * (m + 1) * test;
   }

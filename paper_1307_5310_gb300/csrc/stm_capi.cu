@@ -189,6 +189,7 @@ struct stm_ctx {
   double* tr64 = nullptr;
   float* y32 = nullptr;
   float* tr32 = nullptr;
+  bool no_y32 = false;  // the optional FP32 scratch could not be had or was given back: not tried again
   double* state = nullptr;
   double t = 0.0;
   double* red_partial = nullptr;
@@ -324,12 +325,34 @@ int fail(stm_ctx* c, int code, const std::string& msg) {
   return code;
 }
 
+// Whether a uniform FP32 mesh runs two kernels because that is faster, and could run the single pass.
+bool optional_scratch32(const stm_ctx* c) {
+  return !c->hp && fused_fits(c->P, c->Q) && !single_pass32(c->P, c->Q, c->ne);
+}
+
+// cudaMalloc of memory a call cannot do without.  When there is none left, the optional FP32 scratch
+// is given back first (cudaFree waits for the launches that use it, no captured graph holds it, and
+// later FP32 applies run the single pass).
+template <typename T>
+cudaError_t device_alloc(stm_ctx* c, T** p, size_t bytes) {
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e == cudaErrorMemoryAllocation && c->y32 && optional_scratch32(c)) {
+    cudaGetLastError();
+    cudaFree(c->y32);
+    cudaFree(c->tr32);
+    c->y32 = c->tr32 = nullptr;
+    c->no_y32 = true;
+    e = cudaMalloc((void**)p, bytes);
+  }
+  return e;
+}
+
 int ensure(stm_ctx* c, void** p, size_t* have, size_t need) {
   if (*have >= need) return STM_OK;
   if (*p) cudaFree(*p);
   *p = nullptr;
   *have = 0;
-  if (cudaMalloc(p, need) != cudaSuccess) {
+  if (device_alloc(c, p, need) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, STM_ENOMEM, "device allocation of " + std::to_string(need) + " bytes failed");
   }
@@ -343,7 +366,7 @@ int ensure_scratch(stm_ctx* c, T** y, T** tr) {
   const size_t ny = (size_t)c->n_test;
   const size_t nt = (size_t)c->n_tr;
   T *py = nullptr, *pt = nullptr;
-  if (cudaMalloc((void**)&py, ny * sizeof(T)) != cudaSuccess || cudaMalloc((void**)&pt, nt * sizeof(T)) != cudaSuccess) {
+  if (device_alloc(c, &py, ny * sizeof(T)) != cudaSuccess || device_alloc(c, &pt, nt * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
     if (py) cudaFree(py);  // both or neither: the next call tries again
     return fail(c, STM_ENOMEM, "scratch allocation failed");
@@ -445,25 +468,40 @@ bool needs_scratch(const stm_ctx* c) {
 }
 
 // The scratch of a residual launch (null where it needs none).  Uniform FP32 meshes that are faster in
-// two kernels but also fit the single pass run that one while the scratch cannot be had: on a stream
-// being captured before it exists, or when the allocation fails.
+// two kernels but also fit the single pass (optional_scratch32) must not need memory for that: inside
+// the slab solve (in_solve) they use the FP64 scratch, which the solve's FP64 residuals need anyway and
+// which is idle between them; a direct apply takes FP32 scratch of its own once, given back when other
+// memory is short (device_alloc), and runs the single pass when there is none.  On a stream a caller is
+// capturing it always runs the single pass, so that the graph holds no buffer of the context.
 template <typename T>
-int residual_scratch(stm_ctx* c, T** y, T** tr) {
+int residual_scratch(stm_ctx* c, T** y, T** tr, bool in_solve) {
   *y = *tr = nullptr;
   if (!needs_scratch<T>(c)) return STM_OK;
-  const bool optional = sizeof(T) == 4 && !c->hp && fused_fits(c->P, c->Q);
-  if (optional && !c->y32) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    STM_CK(cudaStreamIsCapturing(c->stream, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return STM_OK;
+  if constexpr (sizeof(T) == 4) {
+    if (optional_scratch32(c)) {
+      if (in_solve) {
+        *y = reinterpret_cast<float*>(c->y64);
+        *tr = reinterpret_cast<float*>(c->tr64);
+        return STM_OK;
+      }
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      STM_CK(cudaStreamIsCapturing(c->stream, &cap));
+      if (cap != cudaStreamCaptureStatusNone) return STM_OK;
+      if (!c->y32 && !c->no_y32) {
+        // relaxed: another thread's capture does not forbid this allocation
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const std::string err = c->err;
+        c->no_y32 = ensure_scratch<float>(c, &c->y32, &c->tr32) != STM_OK;
+        if (c->no_y32) c->err = err;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+      }
+      *y = c->y32;
+      *tr = c->tr32;
+      return STM_OK;
+    }
   }
-  const int rc = scratch<T>(c, y, tr);
-  if (rc && optional) {
-    *y = *tr = nullptr;
-    c->err.clear();
-    return STM_OK;
-  }
-  return rc;
+  return scratch<T>(c, y, tr);
 }
 
 // Upper bound of the residual kernels' grids (grid-stride loops over elements): the launch
@@ -520,7 +558,7 @@ int apply(stm_ctx* c, double dt, const T* um, int um_layout, const T* u0, int u0
           bool pre = false, const int32_t* skip = nullptr) {
   T *y = nullptr, *tr = nullptr;
   {
-    const int rc = residual_scratch<T>(c, &y, &tr);
+    const int rc = residual_scratch<T>(c, &y, &tr, skip != nullptr);  // only the slab solve passes skip
     if (rc) return rc;
   }
   ApplyArgs<T> a{};
@@ -1041,8 +1079,8 @@ int build_load(stm_ctx* c, double t0, double dt, const double** out) {
   }
   const int64_t n = c->n_test;
   if (!c->load64) {
-    if (cudaMalloc(&c->load64, n * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&c->load32, n * sizeof(float)) != cudaSuccess) {
+    if (device_alloc(c, &c->load64, n * sizeof(double)) != cudaSuccess ||
+        device_alloc(c, &c->load32, n * sizeof(float)) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, STM_ENOMEM, "load vector allocation failed");
     }
@@ -1246,8 +1284,8 @@ int build_eta_weights(stm_ctx* c, double dt) {
       w32[6 * e + fc] = (float)w[6 * e + fc];
     }
   if (!c->sw64) {
-    if (cudaMalloc(&c->sw64, w.size() * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&c->sw32, w32.size() * sizeof(float)) != cudaSuccess) {
+    if (device_alloc(c, &c->sw64, w.size() * sizeof(double)) != cudaSuccess ||
+        device_alloc(c, &c->sw32, w32.size() * sizeof(float)) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, STM_ENOMEM, "weight allocation failed");
     }
@@ -1319,7 +1357,7 @@ int ensure_buf(stm_ctx* c, T** p, int64_t* have, int64_t need) {
   if (*p) cudaFree(*p);
   *p = nullptr;
   *have = 0;
-  if (cudaMalloc((void**)p, (size_t)need * sizeof(T)) != cudaSuccess) {
+  if (device_alloc(c, p, (size_t)need * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, STM_ENOMEM, "solver workspace allocation failed");
   }
@@ -2218,7 +2256,7 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
   // b - M x (at most three times) until that is below 1e-15 |b| (the recursively updated
   // residual of CG drifts away from the true one near round-off)
   double* buf = nullptr;
-  if (cudaMalloc(&buf, 6 * (size_t)n * sizeof(double)) != cudaSuccess) {
+  if (device_alloc(c, &buf, 6 * (size_t)n * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, STM_ENOMEM, "projection work vectors");
   }
@@ -2406,16 +2444,18 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
     return rc;
   }
   if (!c->gst) {
-    if (cudaMalloc((void**)&c->gst, sizeof(GmresState)) != cudaSuccess ||
+    if (device_alloc(c, &c->gst, sizeof(GmresState)) != cudaSuccess ||
         cudaMallocHost((void**)&c->h_gst, sizeof(GmresState) + 64) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, STM_ENOMEM, "GMRES state allocation failed");
     }
     STM_CK(cudaMemsetAsync(c->gst, 0, sizeof(GmresState), c->stream));
   }
-  if (mixed) {  // FP32 residual scratch, allocated before any capture
+  {  // residual scratch, allocated before any capture: FP64 first, the FP32 cycles may share it
+    double *y64 = nullptr, *tr64 = nullptr;
     float *y32 = nullptr, *tr32 = nullptr;
-    if ((rc = residual_scratch<float>(c, &y32, &tr32))) return rc;
+    if ((rc = scratch<double>(c, &y64, &tr64))) return rc;
+    if (mixed && (rc = residual_scratch<float>(c, &y32, &tr32, true))) return rc;
   }
   const double* b = nullptr;
   if ((rc = build_load(c, c->t, dt, &b))) return rc;
@@ -2538,7 +2578,8 @@ int32_t stm_dof_layout(stm_ctx* c, int64_t* off_trial, int64_t* off_test, int64_
 template <typename T>
 int autotune_prec(stm_ctx* c, double dt, int reps, std::vector<double>& best_ms) {
   T *U = nullptr, *R = nullptr;
-  if (cudaMalloc(&U, c->n_trial * sizeof(T)) != cudaSuccess || cudaMalloc(&R, c->n_test * sizeof(T)) != cudaSuccess) {
+  if (device_alloc(c, &U, c->n_trial * sizeof(T)) != cudaSuccess ||
+      device_alloc(c, &R, c->n_test * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
     if (U) cudaFree(U);
     return fail(c, STM_ENOMEM, "autotune buffers");
