@@ -29,9 +29,20 @@ struct CurvedTables {
 int launch_metric(int P, const double* X8, const double* eps, const double* mu, int64_t ne, const CurvedTables& ct,
                   double* Gw, double* Pinv, int* bad, cudaStream_t s);
 
+// Launch shape of the curved mass kernel: a CTA takes `epc` elements with all their jobs (a job is one
+// field and temporal mode of an element), or one of `split` shares of one element's jobs (epc = 1), in
+// batches of `jobs`; `parts` threads per coefficient plane, `threads` per CTA, `grid` CTAs.
+struct MassShape {
+  int epc = 0, jobs = 0, split = 0, parts = 0, threads = 0, grid = 0;  // epc = 0: none chosen
+  size_t smem = 0;
+};
+// The shape for ne elements of degree (P, Q) in precision T on the current device; start: with u0.
+template <typename T>
+MassShape mass_shape(int P, int Q, bool start, int64_t ne);
+
 // R[e][f][c][i][s] = mat_f (M_G (u_{i+1} - delta_{i0} u_0))[c][s] for every element (curved_mass.cu).
 template <typename T>
-int launch_mass_curved(int P, int Q, const T* um, int64_t um_es, int64_t um_cs, const T* u0, int64_t u0_es,
+int launch_mass_curved(const MassShape& shape, int P, int Q, const T* um, int64_t um_es, int64_t um_cs, const T* u0, int64_t u0_es,
                        int64_t u0_cs, const T* Gw, const T* eps, const T* mu, const CurvedTables& ct, int64_t ne, T* R,
                        cudaStream_t s, const int32_t* skip = nullptr);
 

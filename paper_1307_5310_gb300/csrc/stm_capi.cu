@@ -277,6 +277,7 @@ struct stm_ctx {
   int* wait_err = nullptr;     // set by the FP32 Krylov kernel if a bounded wait on its copies ran out
   double* el = nullptr;      // per-element energies (curved)
   CurvedTables ct{};
+  MassShape mass_plan[2][2];  // curved mass launch shapes, chosen once: [FP64, FP32][without, with u0]
   // load vector L (Gaussian currents, boundary data g), cached per (t0, dt)
   std::vector<stm_gauss_src> srcs;
   stm_st_field_fn gfn = nullptr;
@@ -749,8 +750,10 @@ int apply(stm_ctx* c, double dt, const T* um, int um_layout, const T* u0, int u0
   }
   if (c->geometry == STM_GEOM_TRILINEAR) {
     // curved: the metric-dependent mass term goes first into R; the residual kernels add the rest
+    MassShape& shape = c->mass_plan[sizeof(T) == 8 ? 0 : 1][a.u0 ? 1 : 0];
+    if (!shape.epc) shape = mass_shape<T>(c->P, c->Q, a.u0 != nullptr, c->ne);
     const int em =
-        launch_mass_curved<T>(c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, curved_ptr<T>(c, 0),
+        launch_mass_curved<T>(shape, c->P, c->Q, a.um, a.um_es, a.um_cs, a.u0, a.u0_es, a.u0_cs, curved_ptr<T>(c, 0),
                               curved_ptr<T>(c, 1), curved_ptr<T>(c, 2), c->ct, c->ne, R, c->stream, skip);
     c->launches += 1;
     if (em) return fail(c, STM_EDEVICE, std::string("curved mass launch: ") + cudaGetErrorString((cudaError_t)em));
@@ -2269,8 +2272,9 @@ int project_curved(stm_ctx* c, double t, stm_field_fn E0, stm_field_fn H0, void*
     *out = c->h_pinned[0];
     return STM_OK;
   };
+  const MassShape shape = mass_shape<double>(P, 1, false, c->ne);
   auto mass = [&](const double* in, double* out) -> int {
-    const int em = launch_mass_curved<double>(P, 1, in, 6LL * N3, N3, nullptr, 0, 0, c->Gw64, c->eps64, c->mu64,
+    const int em = launch_mass_curved<double>(shape, P, 1, in, 6LL * N3, N3, nullptr, 0, 0, c->Gw64, c->eps64, c->mu64,
                                               c->ct, c->ne, out, c->stream);
     c->launches += 1;
     return em ? fail(c, STM_EDEVICE, "projection mass launch") : STM_OK;
