@@ -74,15 +74,17 @@ __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_
 // PARTS: threads per plane in passes A and C.  With two, pass A splits the Gauss columns of a plane
 // between them and pass C the coefficient rows by parity (an even row needs only the sums of a pair of
 // Gauss points, an odd row only the differences), so no operation is done twice.
+// SPLIT: several CTAs may share an element's jobs (FP32 meshes that fill the GPU run without: at p = 0 the
+// unit arithmetic costs 6%).
 // Registers: 128 a thread but for the FP64 planes of N >= 5.
-template <typename T, int P, int PARTS>
+template <typename T, int P, int PARTS, bool SPLIT>
 __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
                                   PARTS == 2 ? (P <= 3 ? 2 : 1) : (sizeof(T) == 4 ? 2 : (P <= 3 ? 4 : 1)))
     k_mass(const T* __restrict__ um, int64_t um_es, int64_t um_cs,
                                               const T* __restrict__ u0, int64_t u0_es, int64_t u0_cs,
                                               const T* __restrict__ Gw, const T* __restrict__ eps,
                                               const T* __restrict__ mu, const MassTab<T, P> tb, int Q, int epc,
-                                              int jobs, uint32_t split, int64_t ne, T* __restrict__ R,
+                                              int jobs, uint32_t split, uint32_t units, int64_t ne, T* __restrict__ R,
                                               const int32_t* skip) {
   if (skip && *skip) return;
   using D = MassDims<T, P>;
@@ -200,13 +202,17 @@ __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
     const T* src = Gw + e0 * 6 * NQ3;
     for (int k = tid; k < nel * 3 * NQ3; k += nt) copy_async<2 * sizeof(T)>(g6 + 2 * k, src + 2 * k);
   };
-  // unit w: batches w % split, w % split + split, ... of the element group w / split
-  // (32-bit: element numbers are, and only meshes of few elements are split)
-  const uint32_t units = (uint32_t)((ne + epc - 1) / epc) * split;
+  // unit w: batches w % split, w % split + split, ... of the element group w / split (32-bit: element
+  // numbers are, and only meshes of few elements are split)
   uint32_t w = blockIdx.x;
-  int64_t e0 = (int64_t)(w / split) * epc;
-  int b0 = (int)(w % split) * jobs, sl = 0;
-  if (w < units) {
+  int64_t e0 = (int64_t)w * epc;
+  int b0 = 0, sl = 0;
+  auto unit = [&](uint32_t u, int64_t& e, int& b) {
+    e = (int64_t)(u / split) * epc;
+    b = (int)(u % split) * jobs;
+  };
+  if constexpr (SPLIT) unit(w, e0, b0);
+  if (SPLIT ? w < units : e0 < ne) {
     fetch(e0, b0, 0);
     fetch_metric(e0);
   }
@@ -219,18 +225,22 @@ __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
     __syncthreads();
     op = PassOps<T>{tab[2 * N * (H + 1)], tab[2 * N * (H + 1) + 1], tab[2 * N * (H + 1) + 2]};
   }
-  while (w < units) {
+  while (SPLIT ? w < units : e0 < ne) {
     {
       const int nel = (int)(ne - e0 < epc ? ne - e0 : epc), total = nel * jpe;
       const int nj = total - b0 < jobs ? total - b0 : jobs;
       // the batch after this one
       uint32_t w1 = w;
       int64_t e1 = e0;
-      int b1 = b0 + (int)split * jobs;
+      int b1 = b0 + (SPLIT ? (int)split : 1) * jobs;
       if (b1 >= total) {
-        w1 = w + gridDim.x;
-        e1 = (int64_t)(w1 / split) * epc;
-        b1 = (int)(w1 % split) * jobs;
+        if constexpr (SPLIT) {
+          w1 = w + gridDim.x;
+          unit(w1, e1, b1);
+        } else {
+          b1 = 0;
+          e1 = e0 + (int64_t)gridDim.x * epc;
+        }
       }
       copy_async_wait();
       __syncthreads();
@@ -282,14 +292,16 @@ __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
         }
       }
       __syncthreads();
-      if (w1 < units) fetch(e1, b1, sl ^ 1);
+      const bool more = SPLIT ? w1 < units : e1 < ne;
+      if (more) fetch(e1, b1, sl ^ 1);
       // z, the metric, z back: one Gauss column, planes (c, l) PT apart.  BP = 3: a thread per column
       // and result component (c0), each with its own forward contractions; the column is read by all
       // three before one of them stores
       const int per = nt / BP;
       for (int k0 = 0; k0 < nj * NQ2; k0 += per) {
         const int k = k0 + tid / BP, c0 = BP == 1 ? 0 : tid % BP;
-        const bool mine = tid < per * BP && k < nj * NQ2;
+        const bool mine = BP == 1 || (tid < per * BP && k < nj * NQ2);
+        if (BP == 1 && k >= nj * NQ2) break;
         const int jl = k / NQ2, col = k - jl * NQ2;
         const T* G = g6 + (epc > 1 ? (b0 + jl) / jpe : 0) * 6 * NQ3 + col;
         T* B = tb2 + jl * 3 * N * PT + col;
@@ -339,7 +351,7 @@ __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
           for (int l = 0; l < N; ++l) B[((c0 + c) * N + l) * PT] = a[c][l];
       }
       __syncthreads();
-      if (w1 < units && w1 != w) fetch_metric(e1);
+      if (more && (SPLIT ? w1 != w : b1 == 0)) fetch_metric(e1);
       {
         // rows of this thread: all N, or with two parts k = 2 kk + part
         constexpr int NK = PARTS == 1 ? N : (N + 1) / 2;
@@ -418,8 +430,8 @@ __global__ void __launch_bounds__(MassDims<T, P>::MAXT * PARTS,
 // A mesh that fills at least half of the co-resident CTAs takes the shape with the least idle lanes in
 // passes A/C (one plane per thread) and B (columns over the same threads) within a budget of shared
 // memory per CTA.  Smaller meshes wait for the chain of one CTA, and the FP64 planes of p >= 5 leave one
-// or two CTAs of 32 to 128 threads per SM, with the FP64 pipe idle at every barrier: they take the
-// shape with the least estimated time, over elements per CTA, jobs per batch, units per element,
+// or two CTAs of 32 to 128 threads per SM, with the FP64 pipe idle at every barrier: both (FP32 of p >= 3
+// excepted, whose chains are short) take the shape with the least estimated time, over elements per CTA, jobs per batch, units per element,
 // threads per plane and block sizes.  The estimate: the busiest SM runs `rounds` times c units of nb
 // batches; a batch takes x us alone (FP64: 64 clocks per warp instruction on each of an SM's four
 // partitions, plus the rows of the copies) and y us of the SM's shared pipes.  Its constants are fitted
@@ -441,9 +453,11 @@ MassShape mass_shape_p(int Q, bool start, int64_t ne) {
     cudaGetLastError();
   static std::atomic<uint64_t> configured_devices{0};
   once_per_device(configured_devices, [&] {
-    cudaFuncSetAttribute(k_mass<T, P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    cudaFuncSetAttribute(k_mass<T, P, 1, F64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if constexpr (F64)
-      cudaFuncSetAttribute(k_mass<T, P, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+      cudaFuncSetAttribute(k_mass<T, P, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    else if constexpr (P <= 2)
+      cudaFuncSetAttribute(k_mass<T, P, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   });
   auto smem = [&](int epc, int jobs) {
     return sizeof(T) * ((size_t)epc * 6 * D::NQ3 + (start ? (size_t)(jobs <= Q ? 1 : 2 * epc) * 3 * N * D::PV : 0) +
@@ -453,10 +467,10 @@ MassShape mass_shape_p(int Q, bool start, int64_t ne) {
     int occ = 0;
     cudaError_t e;
     if constexpr (F64)
-      e = parts == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 2>, threads, sm)
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 1>, threads, sm);
+      e = parts == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 2, true>, threads, sm)
+                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 1, F64>, threads, sm);
     else
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 1>, threads, sm);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_mass<T, P, 1, F64>, threads, sm);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess ? occ : 0;
   };
@@ -471,6 +485,7 @@ MassShape mass_shape_p(int Q, bool start, int64_t ne) {
     for (int jobs = 1; jobs <= epc * 2 * Q && jobs <= kMassJobs; ++jobs) {
       const int planes = 3 * N * jobs, threads = (planes + 31) / 32 * 32;
       if (!divides(epc, jobs) || threads > D::MAXT || smem(epc, jobs) > D::WANT) continue;
+      if (start && jobs <= Q && smem(epc, jobs) + sizeof(T) * 3 * N * D::PV > D::WANT) continue;  // room for both fields' starts
       const int cols = D::NQ2 * jobs, rounds = (cols + threads - 1) / threads;
       const double a = (double)planes / threads, b = (double)cols / (rounds * threads);
       // small CTAs spend their time between barriers
@@ -482,6 +497,7 @@ MassShape mass_shape_p(int Q, bool start, int64_t ne) {
     }
   const int occ = resident(1, best.threads, best.smem);
   best.grid = grid(best, occ);
+  if (!F64 && P >= 3 && best_score >= 0) return best;
   if (!(F64 && P >= 5) && best_score >= 0 && 2 * ((ne + best.epc - 1) / best.epc) >= (int64_t)occ * sms) return best;
   // least estimated time
   const double fwd = H * N + (N > 1 ? H : 0) + C * ((N + 1) / 2 - 1);  // operations of a line, there and back
@@ -503,7 +519,7 @@ MassShape mass_shape_p(int Q, bool start, int64_t ne) {
           const double rows = (double)((3 * jobs + w - 1) / w) * ((D::N3 + 31) / 32);
           const double metric = (double)((epc * 3 * D::NQ3 + threads - 1) / threads);
           for (int split = 1; split <= batches; ++split) {
-            if (batches % split) continue;
+            if (batches % split || (!F64 && P >= 3 && split > 1)) continue;  // (no such instance)
             const MassShape s{epc, jobs, split, parts, threads, 0, smem(epc, jobs)};
             const int64_t units = (ne + epc - 1) / epc * split;
             const int g = grid(s, occ);
@@ -545,16 +561,20 @@ int mass_p(const MassShape& sh, int Q, const T* um, int64_t um_es, int64_t um_cs
     }
     tb.L[j][H] = ((P + 2) & 1) && !(j & 1) ? (T)ct.Lq[j][H] : T(0);
   }
+  const uint32_t units = (uint32_t)((ne + sh.epc - 1) / sh.epc * sh.split);
   // persistent over the units, one wave of co-resident CTAs (a skipped launch costs one wave)
   auto go = [&](auto kernel) {
     kernel<<<sh.grid, sh.threads, sh.smem, s>>>(um, um_es, um_cs, u0, u0_es, u0_cs, Gw, eps, mu, tb, Q, sh.epc, sh.jobs,
-                                                (uint32_t)sh.split, ne, R, skip);
+                                                (uint32_t)sh.split, units, ne, R, skip);
   };
   if constexpr (sizeof(T) == 8) {
-    if (sh.parts == 2) go(k_mass<T, P, 2>);
-    else go(k_mass<T, P, 1>);
+    if (sh.parts == 2) go(k_mass<T, P, 2, true>);
+    else go(k_mass<T, P, 1, true>);
+  } else if constexpr (P <= 2) {
+    if (sh.split > 1) go(k_mass<T, P, 1, true>);
+    else go(k_mass<T, P, 1, false>);
   } else {
-    go(k_mass<T, P, 1>);
+    go(k_mass<T, P, 1, false>);
   }
   return (int)cudaGetLastError();
 }
