@@ -447,6 +447,18 @@ struct ApplyShape {
   static constexpr size_t smem = sizeof(T) * 2 * NF * 3 * Q * N3;
 };
 
+// The same for k_apply.  Uniform FP32 meshes of high degree are bound by their loads: with the largest
+// block they keep 40 registers a thread, so that three blocks share an SM where shared memory has room
+// for three (53 registers leave two).  FP32 residual, two blocks -> three: 9^3 bricks p = 7, q = 6
+// 176 -> 148 us; with the affine mass's loads together, 13^3 affine elements p = q = 5 168 -> 119 us.
+template <typename T, int P, int Q, bool HP>
+__host__ __device__ constexpr int apply_min_blocks() {
+  return sizeof(T) == 4 && !HP && residual_max_threads(P, Q) == 512 &&
+                 3 * (ApplyShape<T, P, Q>::smem + 3072) <= 228 * 1024
+             ? 3
+             : residual_min_blocks(P, Q);
+}
+
 // Position of the nonzero D[a][b] (d_nz) of an N x N table in row order; d_count<N>(N, 0) of them.
 template <int N>
 __host__ __device__ constexpr int d_count(int a, int b) {
@@ -474,7 +486,7 @@ struct LineTab {
 // modes before the first product.  64^3 bricks, p = 4, q = 3, FP64: 10.27 -> 8.55 ms; without the
 // trace loads of the line passes it takes 7.5 ms, with all memory traffic hitting L2 8.4 ms.
 template <typename T, int P, int Q, bool HP, bool TR = false>
-__global__ void __launch_bounds__(residual_max_threads(P, Q), residual_min_blocks(P, Q)) k_apply(ApplyArgs<T> A) {
+__global__ void __launch_bounds__(residual_max_threads(P, Q), apply_min_blocks<T, P, Q, HP>()) k_apply(ApplyArgs<T> A) {
   if (A.skip && *A.skip) return;
   constexpr int N = P + 1, N2 = N * N, N3 = N2 * N;
   constexpr int NF = ApplyShape<T, P, Q>::NF;
@@ -602,19 +614,40 @@ __global__ void __launch_bounds__(residual_max_threads(P, Q), residual_min_block
           sym3_row(A.mass3 + (e * 2 + f) * 6, cc, mr);
           const T* uf = A.um + ad.um + (int64_t)(f * 3) * ad.um_cs + s;
           T* Rr = Rs + fl * FB + cc * Q * N3 + s;
-#pragma unroll 1
-          for (int i = 0; i < Q; ++i) {
-            T v = mr[0] * uf[i * N3];
-            v = fma(mr[1], uf[ad.um_cs + i * N3], v);
-            v = fma(mr[2], uf[2 * ad.um_cs + i * N3], v);
-            if (i == 0 && A.u0) {
+          if constexpr (sizeof(T) == 4) {
+            T v[Q];  // the modes of a component load together
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v[i] = mr[0] * uf[i * N3];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v[i] = fma(mr[1], uf[ad.um_cs + i * N3], v[i]);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v[i] = fma(mr[2], uf[2 * ad.um_cs + i * N3], v[i]);
+            if (A.u0) {
               const T* u0f = A.u0 + ad.u0 + (int64_t)(f * 3) * ad.u0_cs + s;
-              v = fma(-mr[0], u0f[0], v);
-              v = fma(-mr[1], u0f[ad.u0_cs], v);
-              v = fma(-mr[2], u0f[2 * ad.u0_cs], v);
+              v[0] = fma(-mr[0], u0f[0], v[0]);
+              v[0] = fma(-mr[1], u0f[ad.u0_cs], v[0]);
+              v[0] = fma(-mr[2], u0f[2 * ad.u0_cs], v[0]);
             }
-            if (A.b) v -= A.b[test_ofs<Q, N3, TR>(rk, f, (cc * Q + i) * N3 + s, QE)];
-            Rr[i * N3] = v;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+              if (A.b) v[i] -= A.b[test_ofs<Q, N3, TR>(rk, f, (cc * Q + i) * N3 + s, QE)];
+              Rr[i * N3] = v[i];
+            }
+          } else {
+#pragma unroll 1
+            for (int i = 0; i < Q; ++i) {
+              T v = mr[0] * uf[i * N3];
+              v = fma(mr[1], uf[ad.um_cs + i * N3], v);
+              v = fma(mr[2], uf[2 * ad.um_cs + i * N3], v);
+              if (i == 0 && A.u0) {
+                const T* u0f = A.u0 + ad.u0 + (int64_t)(f * 3) * ad.u0_cs + s;
+                v = fma(-mr[0], u0f[0], v);
+                v = fma(-mr[1], u0f[ad.u0_cs], v);
+                v = fma(-mr[2], u0f[2 * ad.u0_cs], v);
+              }
+              if (A.b) v -= A.b[test_ofs<Q, N3, TR>(rk, f, (cc * Q + i) * N3 + s, QE)];
+              Rr[i * N3] = v;
+            }
           }
         }
       } else {
