@@ -254,17 +254,23 @@ struct PassOps {
 
 // Default block of the two-kernel passes, by the element's work per pass: small blocks, so that many
 // elements are in different phases (loads, mass rows, line passes, stores) on an SM, as long as
-// the lines of a pass keep their warps busy.  The lines lie where the autotuner's sweep over
-// p = 1..7, q = 1..4 (FP64, uniform and hp meshes, 64..512 threads) changes its choice; at p = 4,
-// q = 3 (64^3 bricks) 128 threads take 8.55 ms per k_apply against 8.91 ms for 256.  A mesh (or
-// class) of at most two elements per SM (152) waits for one element's own chain of loads, passes
-// and barriers instead: at least 256 threads there (4^3 elements, p = 2, q = 1: 11.6 us per apply
-// against 14.4 us for 64).
-constexpr int residual_default_block(int P, int Q, int64_t n_elem) {
-  const int w = Q * (P + 1) * (P + 1) * (P + 1);
+// the lines of a pass keep their warps busy.  The lines lie where the autotuner (stm_autotune) changes
+// its choice over p = 1..7, q = 1..4 (FP64, uniform and hp meshes, 64..512 threads); at p = 4,
+// q = 3 (64^3 bricks) 128 threads take 8.55 ms per k_apply against 8.91 ms for 256.  A uniform mesh
+// of few elements per SM (152) waits for the elements' own chains of loads, passes and barriers
+// instead: the largest block up to two elements per SM, at least 256 threads up to four, 128 up to
+// eight.  The classes of an uneven mesh share the SMs with one another, so only a class of at most two
+// elements per SM takes 256 (12^3 elements, p = q = 1, N_K in {1, 2, 4}: 28.8 us a residual, with the
+// uniform mesh's lines 45.1).  FP64 residual of bricks with the block by work alone -> this rule, us: 5^3 p = 6, q = 2
+// 29.0 -> 24.9, p = 5, q = 3 24.8 -> 22.8; 7^3 p = 4, q = 1 24.8 -> 16.6, p = 2, q = 6 26.9 -> 18.8;
+// 9^3 p = 4, q = 1 26.9 -> 23.0, p = 2, q = 6 31.0 -> 26.8.
+constexpr int residual_default_block(int P, int Q, int64_t n_elem, bool uniform = true) {
+  const int w = Q * (P + 1) * (P + 1) * (P + 1), most = residual_max_threads(P, Q);
   const int t = w <= 200 ? 64 : (w <= 380 ? 128 : (w <= 700 ? 256 : 512));
-  const int b = n_elem <= 2 * 152 && t < 256 ? 256 : t;
-  return b < residual_max_threads(P, Q) ? b : residual_max_threads(P, Q);
+  const int few = n_elem <= 2 * 152 ? (uniform ? most : 256)
+                                    : (!uniform || n_elem > 8 * 152 ? 64 : (n_elem <= 4 * 152 ? 256 : 128));
+  const int b = few > t ? few : t;
+  return b < most ? b : most;
 }
 
 // Blocks per SM the compiler leaves registers for: 64 registers a thread at the largest block.

@@ -1882,7 +1882,7 @@ int32_t stm_create(stm_ctx** out, const stm_mesh* m, const stm_opts* o) {
         for (int lk = 0; lk < 4 && okh; ++lk) {
           const auto& L = lists[(pp * (kMaxQ + 1) + qq) * 4 + lk];
           if (L.empty()) continue;
-          stm_ctx::Class cl{pp, qq, (int64_t)L.size(), nullptr, residual_default_block(pp, qq, (int64_t)L.size())};
+          stm_ctx::Class cl{pp, qq, (int64_t)L.size(), nullptr, residual_default_block(pp, qq, (int64_t)L.size(), false)};
           cl.NK = 1 << lk;
           okh = cudaMalloc(&cl.elist, L.size() * sizeof(int32_t)) == cudaSuccess;
           if (okh) cudaMemcpy(cl.elist, L.data(), L.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
