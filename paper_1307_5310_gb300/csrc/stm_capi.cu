@@ -2498,10 +2498,11 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
   // read of the device state: the stop test, the iteration count and the error status
   bool done = false;
   const int per = c->profiling ? 1 : std::max(1, (int)c->opts.cycles_per_launch);
-  const int max_launches = c->opts.max_it + 2;  // every cycle but the last makes >= 1 iteration
+  // every cycle but the last makes >= 1 iteration; at least one launch reads the state (max_it <= 0)
+  const int64_t max_launches = std::max<int64_t>(1, (int64_t)c->opts.max_it + 2);
   int* h_err = reinterpret_cast<int*>(c->h_gst + 1);  // the Krylov kernel's wait flag, read with the state
   if ((rc = run_cycles(c, dt, b, mixed, ldv, 0))) return rc;
-  for (int cyc = 0; cyc < max_launches; ++cyc) {
+  for (int64_t cyc = 0; cyc < max_launches; ++cyc) {
     if ((rc = run_cycles(c, dt, b, mixed, ldv, per))) return rc;
     STM_CK(cudaMemcpyAsync(c->h_gst, st, sizeof(GmresState), cudaMemcpyDeviceToHost, c->stream));
     STM_CK(cudaMemcpyAsync(h_err, c->wait_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
