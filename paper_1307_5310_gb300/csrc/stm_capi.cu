@@ -348,6 +348,21 @@ cudaError_t device_alloc(stm_ctx* c, T** p, size_t bytes) {
   return e;
 }
 
+// Both of a pair of buffers or neither, so that a call after a failed one starts over.
+template <typename A, typename B>
+bool device_alloc_pair(stm_ctx* c, A** a, size_t na, B** b, size_t nb) {
+  A* pa = nullptr;
+  B* pb = nullptr;
+  if (device_alloc(c, &pa, na * sizeof(A)) != cudaSuccess || device_alloc(c, &pb, nb * sizeof(B)) != cudaSuccess) {
+    cudaGetLastError();
+    if (pa) cudaFree(pa);
+    return false;
+  }
+  *a = pa;
+  *b = pb;
+  return true;
+}
+
 int ensure(stm_ctx* c, void** p, size_t* have, size_t need) {
   if (*have >= need) return STM_OK;
   if (*p) cudaFree(*p);
@@ -364,16 +379,8 @@ int ensure(stm_ctx* c, void** p, size_t* have, size_t need) {
 template <typename T>
 int ensure_scratch(stm_ctx* c, T** y, T** tr) {
   if (*y) return STM_OK;
-  const size_t ny = (size_t)c->n_test;
-  const size_t nt = (size_t)c->n_tr;
-  T *py = nullptr, *pt = nullptr;
-  if (device_alloc(c, &py, ny * sizeof(T)) != cudaSuccess || device_alloc(c, &pt, nt * sizeof(T)) != cudaSuccess) {
-    cudaGetLastError();
-    if (py) cudaFree(py);  // both or neither: the next call tries again
+  if (!device_alloc_pair(c, y, (size_t)c->n_test, tr, (size_t)c->n_tr))
     return fail(c, STM_ENOMEM, "scratch allocation failed");
-  }
-  *y = py;
-  *tr = pt;
   return STM_OK;
 }
 
@@ -1082,11 +1089,8 @@ int build_load(stm_ctx* c, double t0, double dt, const double** out) {
   }
   const int64_t n = c->n_test;
   if (!c->load64) {
-    if (device_alloc(c, &c->load64, n * sizeof(double)) != cudaSuccess ||
-        device_alloc(c, &c->load32, n * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
+    if (!device_alloc_pair(c, &c->load64, n, &c->load32, n))
       return fail(c, STM_ENOMEM, "load vector allocation failed");
-    }
   }
   if (c->hp) {
     // uneven degrees or N_K: the host callbacks (J, g) are sampled and projected on the
@@ -1287,11 +1291,8 @@ int build_eta_weights(stm_ctx* c, double dt) {
       w32[6 * e + fc] = (float)w[6 * e + fc];
     }
   if (!c->sw64) {
-    if (device_alloc(c, &c->sw64, w.size() * sizeof(double)) != cudaSuccess ||
-        device_alloc(c, &c->sw32, w32.size() * sizeof(float)) != cudaSuccess) {
-      cudaGetLastError();
+    if (!device_alloc_pair(c, &c->sw64, w.size(), &c->sw32, w32.size()))
       return fail(c, STM_ENOMEM, "weight allocation failed");
-    }
   }
   STM_CK(cudaMemcpy(c->sw64, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice));
   STM_CK(cudaMemcpy(c->sw32, w32.data(), w32.size() * sizeof(float), cudaMemcpyHostToDevice));
@@ -2448,11 +2449,14 @@ int32_t stm_slab_solve(stm_ctx* c, double dt, stm_solve_report* rep) {
     return rc;
   }
   if (!c->gst) {
-    if (device_alloc(c, &c->gst, sizeof(GmresState)) != cudaSuccess ||
+    GmresState* gst = nullptr;
+    if (device_alloc(c, &gst, sizeof(GmresState)) != cudaSuccess ||
         cudaMallocHost((void**)&c->h_gst, sizeof(GmresState) + 64) != cudaSuccess) {
       cudaGetLastError();
+      if (gst) cudaFree(gst);
       return fail(c, STM_ENOMEM, "GMRES state allocation failed");
     }
+    c->gst = gst;
     STM_CK(cudaMemsetAsync(c->gst, 0, sizeof(GmresState), c->stream));
   }
   {  // residual scratch, allocated before any capture: FP64 first, the FP32 cycles may share it

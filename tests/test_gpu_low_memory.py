@@ -131,6 +131,23 @@ L.mem_limit(L.mem_total() - own + 12 * test + 65536)
 s.set_source_gauss(SRC)
 assert apply32(s, RL) < 2e-6
 """,
+    # the FP64 half of the load fits, the FP32 half does not: refused, and again, until there is room
+    "load_in_halves": r"""
+s = slab()
+s.residual_apply(U, R, 0.0, dt)
+s.set_source_gauss(SRC)
+L.mem_limit(L.mem_total() + 8 * test + 4096)
+n = L.mem_total()
+for k in range(2):
+    try:
+        apply32(s, RL)
+        assert False, "fits"
+    except stm.StmError as e:
+        assert e.code == stm.STM_ENOMEM, e
+    assert L.mem_total() == n
+L.mem_limit(-1)
+assert apply32(s, RL) < 2e-6
+""",
     # no room at all: the apply runs without scratch, asks for it once and leaves no error text
     "apply_without_room": r"""
 s = slab()
