@@ -860,9 +860,9 @@ def run_ours(args):
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     fp64_peak = 4.0 * sms * sm_mhz * 1e6 / 1e12  # 2 FP64 FMA / clock / SM
     ach = fl_apply * ne / (apply_ms / 1e3) / 1e12
-    # DRAM bytes per k_apply launch from one ncu capture of the 32^3 case (1.936 GB read + 0.572 GB
+    # DRAM bytes per k_apply launch from one ncu capture of the 32^3 case (1.880 GB read + 0.560 GB
     # written), scaled by the element count to this workload; valid for p=4, q=3 on 64^3 only
-    traffic = 2.507e9 * ne / 32 ** 3 if (args.n, args.p, args.q) == (64, 4, 3) else None
+    traffic = 2.440e9 * ne / 32 ** 3 if (args.n, args.p, args.q) == (64, 4, 3) else None
     try:  # context: the FP64 FMA rate this GPU reaches in a register-only kernel, measured live
         probe = stm.fp64_probe()
     except Exception:  # reported as missing, never replaced

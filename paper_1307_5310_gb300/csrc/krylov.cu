@@ -563,14 +563,13 @@ __global__ void k_precond(S* __restrict__ z, const S* __restrict__ v, const S* _
 // vectors are far larger than L2, so this is bound by HBM: 32^3 elements, p = 4, q = 3, ten FP32
 // columns 1.01 -> 0.64 ms.
 template <typename S, typename X, int K, bool Small>
-__global__ void k_precond_combine(X* __restrict__ x, const S* __restrict__ V, int64_t ldv, Coef16 y,
+__global__ void k_precond_combine(X* __restrict__ x, const S* __restrict__ V, int64_t ldv,
                                   const S* __restrict__ inv, int64_t blk, int64_t n, const GmresState* st) {
-  // with st: k and the coefficients come from the device state (K is the largest k)
-  const int kk = st ? st->k : K;
+  const int kk = st->k;  // K is the largest
   if (kk <= 0) return;
   S yy[K > 0 ? K : 1];
 #pragma unroll
-  for (int i = 0; i < K; ++i) yy[i] = (S)(st ? st->yc[i] : y.c[i]);
+  for (int i = 0; i < K; ++i) yy[i] = (S)st->yc[i];
   using VS = typename Vec<S>::T;
   using VX = typename Vec<X>::T;
   constexpr int WS = Vec<S>::W, WX = Vec<X>::W, GS = 4 / WS, GX = 4 / WX;
@@ -656,11 +655,11 @@ inline int red_grid(F kernel, int64_t nv, std::atomic<int>* cache) {
 }
 
 template <typename S, typename X, int K>
-void combine_k(X* x, const S* V, int64_t ldv, const Coef16& y, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
+void combine_k(X* x, const S* V, int64_t ldv, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
                const GmresState* st) {
   const int g = grid_for((n + 3) / 4);
-  if (small(n)) k_precond_combine<S, X, K, true><<<g, kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
-  else k_precond_combine<S, X, K, false><<<g, kRedThreads, 0, s>>>(x, V, ldv, y, inv, blk, n, st);
+  if (small(n)) k_precond_combine<S, X, K, true><<<g, kRedThreads, 0, s>>>(x, V, ldv, inv, blk, n, st);
+  else k_precond_combine<S, X, K, false><<<g, kRedThreads, 0, s>>>(x, V, ldv, inv, blk, n, st);
 }
 
 #define STM_SWITCH_K(k, CALL)  \
@@ -759,10 +758,10 @@ void precond_apply(S* z, const S* v, const S* inv, int64_t blk, int64_t n, cudaS
 }
 
 template <typename S, typename X>
-void precond_combine(X* x, const S* V, int64_t ldv, int k, const Coef16& y, const S* inv, int64_t blk, int64_t n,
-                     cudaStream_t s, const GmresState* st) {
-#define STM_CB(K) combine_k<S, X, K>(x, V, ldv, y, inv, blk, n, s, st)
-  STM_SWITCH_K(k, STM_CB)
+void precond_combine(X* x, const S* V, int64_t ldv, int m, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
+                     const GmresState* st) {
+#define STM_CB(K) combine_k<S, X, K>(x, V, ldv, inv, blk, n, s, st)
+  STM_SWITCH_K(m, STM_CB)
 #undef STM_CB
 }
 
@@ -789,13 +788,10 @@ template void precond_apply<double>(double*, const double*, const double*, int64
                                     const int32_t*);
 template void precond_apply<float>(float*, const float*, const float*, int64_t, int64_t, cudaStream_t,
                                    const int32_t*);
-template void precond_combine<double, double>(double*, const double*, int64_t, int, const Coef16&, const double*,
-                                              int64_t, int64_t, cudaStream_t, const GmresState*);
-template void precond_combine<float, double>(double*, const float*, int64_t, int, const Coef16&, const float*,
-                                             int64_t, int64_t, cudaStream_t, const GmresState*);
-template void precond_combine<float, float>(float*, const float*, int64_t, int, const Coef16&, const float*, int64_t,
-                                            int64_t, cudaStream_t, const GmresState*);
+template void precond_combine<double, double>(double*, const double*, int64_t, int, const double*, int64_t, int64_t,
+                                              cudaStream_t, const GmresState*);
+template void precond_combine<float, double>(double*, const float*, int64_t, int, const float*, int64_t, int64_t,
+                                             cudaStream_t, const GmresState*);
 template void convert<float, double>(float*, const double*, int64_t, cudaStream_t, const int32_t*);
-template void convert<double, float>(double*, const float*, int64_t, cudaStream_t, const int32_t*);
 
 }  // namespace stm

@@ -1,10 +1,11 @@
 // Vector kernels of the per-slab GMRES solve (Sec. 5.4) and the discrete
 // energy (Eq. stability:energydef).  Storage type S is double or float.
-// Reductions use a fixed grid and a fixed summation order, so results are
-// bitwise reproducible run to run.  With S = double every product and sum is
-// FP64.  With S = float (the inner solve of the mixed-precision path) each
-// thread sums products of 8 consecutive entries in FP32 and accumulates those
-// partial sums in FP64; the grid and block reductions are FP64.
+// Reductions use a fixed summation order on a grid that follows from the vector
+// length and the device, so results are bitwise reproducible run to run on one
+// kind of device.  With S = double every product and sum is FP64.  With
+// S = float (the inner solve of the mixed-precision path) each thread sums the 16
+// products of four 16-byte chunks, a grid stride apart, in FP32 and accumulates
+// those partial sums in FP64; the grid and block reductions are FP64.
 //
 // The last block of a reduction to arrive sums the grid's partials and takes the scalar step that
 // needs them (Gram-Schmidt coefficients, Givens rotation, stop tests, triangular solve), so an
@@ -36,7 +37,7 @@ struct GmresState {
   double cc[kMaxDots];            // Gram-Schmidt coefficients of the current iteration
   double yc[kMaxDots];            // combination coefficients at the end of the cycle
   double red[4];                  // reduction results: 0 |R|^2, 1 |S R|^2, 2 |start vector|^2
-  double before, after;           // |W|^2 before and after the update (DGKS test)
+  double before;                  // |W|^2 before the update (DGKS test)
   double ref;                     // |R(U with unknowns 0)| of the slab (stop test R6)
   double tol;                     // relative target (exact solve) or eta budget (inexact)
   double tol_abs;                 // this cycle's stop threshold on |g|
@@ -69,11 +70,10 @@ template <typename S>
 void precond_apply(S* z, const S* v, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
                    const int32_t* skip = nullptr);
 
-// x[n] += inv[n / blk] * sum_{i<k} y[i] V[i*ldv + n].  With st non-null, k and y are
-// read from the device state (st->k, st->yc) and k is the largest count.
+// x[n] += inv[n / blk] * sum_{i < st->k} st->yc[i] V[i*ldv + n], st->k <= m.
 template <typename S, typename X>
-void precond_combine(X* x, const S* V, int64_t ldv, int k, const Coef16& y, const S* inv, int64_t blk, int64_t n,
-                     cudaStream_t s, const GmresState* st = nullptr);
+void precond_combine(X* x, const S* V, int64_t ldv, int m, const S* inv, int64_t blk, int64_t n, cudaStream_t s,
+                     const GmresState* st);
 
 // ---- device-side GMRES: reductions whose last block takes the scalar step that follows ----
 // Each launch is skipped on the device once the cycle (st->skip) or the slab (st->halt) has stopped.

@@ -1353,7 +1353,7 @@ int launch_residual_pq(const ApplyArgs<T>& args, cudaStream_t s, int grid, const
   // kernel attributes are per device: set them once on every device this instantiation launches on
   static std::atomic<uint64_t> configured_devices{0};
   // the dynamic shared-memory limit is set for every size: static shared memory (k_prep's
-  // folded coefficients, k_apply's face cache) counts against the same 48 KB default
+  // coefficients, k_apply's tables and face cache) counts against the same 48 KB default
   once_per_device(configured_devices, [&] {
     cudaFuncSetAttribute(k_prep<T, P, Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_prep);
     cudaFuncSetAttribute(k_prep<T, P, Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_prep);

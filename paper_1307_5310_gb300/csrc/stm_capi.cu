@@ -1320,7 +1320,7 @@ void scale_blocks(stm_ctx* c, S* v, const S* w, int64_t n, const int32_t* skip =
 // the Hessenberg column, the Givens rotations and the stop test live in the device
 // state c->gst, and every kernel of an iteration is skipped once the cycle has stopped.
 // The basis is kept unnormalised: v_i = V_i / alpha_i (alpha_i signed), V[0] holds the
-// start vector (set up by gmres_cycle_init).  Classical Gram-Schmidt (one fused dot pass,
+// start vector (its scale set by the stop test of launch_check, or by gmres_start32).  Classical Gram-Schmidt (one fused dot pass,
 // one fused update + norm pass), with an optional second pass when the norm drops below
 // 1/sqrt(2) of its value before the update.  At the end st->yc holds the coefficients
 // such that the correction is P^{-1} sum_{i<k} yc[i] V[i].
@@ -1416,7 +1416,7 @@ int launch_cycle(stm_ctx* c, double dt, const double* b, bool mixed, int64_t ldv
                                                nullptr, st);
     else if (c->hp) combine_hp<double, double>(c->x, c->V, ldv, m, Coef16{}, c->inv64, c->off_test, c->pq, c->ne,
                                                c->stream, st);
-    else precond_combine<double, double>(c->x, c->V, ldv, m, Coef16{}, c->inv64, qn3, n, c->stream, st);
+    else precond_combine<double, double>(c->x, c->V, ldv, m, c->inv64, qn3, n, c->stream, st);
   } else {
     // FP32 inner GMRES(m) cycle on A d = r, started from the rounded FP64 residual; the inner
     // target is the outer one or what FP32 can resolve (1e-6 of the start), whichever is larger
@@ -1427,7 +1427,7 @@ int launch_cycle(stm_ctx* c, double dt, const double* b, bool mixed, int64_t ldv
                                               nullptr, st);
     else if (c->hp) combine_hp<float, double>(c->x, c->V32, ldv, m, Coef16{}, c->inv32, c->off_test, c->pq, c->ne,
                                               c->stream, st);
-    else precond_combine<float, double>(c->x, c->V32, ldv, m, Coef16{}, c->inv32, qn3, n, c->stream, st);
+    else precond_combine<float, double>(c->x, c->V32, ldv, m, c->inv32, qn3, n, c->stream, st);
   }
   c->launches += 1;
   return launch_check(c, dt, b, mixed);
